@@ -358,16 +358,39 @@ __device__ __forceinline__ int nth_set_bit(unsigned m, int k)
     return pos;
 }
 
+// One update job of pooled_update: the state and the hit parked at column st of the block's
+// planes.  Out of line, so that the update's registers and the scan's do not meet in one
+// allocation: the kernel around the call keeps the contractions it has without it.
+template <class U, class R, int T> __device__ __noinline__ void pooled_job(float *st, bool disk)
+{
+    R p[6], P[21];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) p[k] = st[k * T];
+#pragma unroll
+    for (int k = 0; k < 21; ++k) P[k] = st[(6 + k) * T];
+    const R hx = st[27 * T], hy = st[28 * T], hz = st[29 * T], vu = st[30 * T], vv = st[31 * T];
+    R dc2 = R(0);
+    if (disk)
+        state_update<U, R, true>(p, P, hx, hy, hz, vu, vv, &dc2);
+    else
+        state_update<U, R, false>(p, P, hx, hy, hz, vu, vv, &dc2);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) st[k * T] = p[k];
+#pragma unroll
+    for (int k = 0; k < 21; ++k) st[(6 + k) * T] = P[k];
+}
+
 // The Kalman updates of a block's candidates, packed into as few warps as they fill (mixed
-// precision).  The update is the kernel's only double-precision work, and the double-precision
-// pipe spends the same time on a warp instruction whatever its active lanes; a warp's own
-// candidates with a hit (about 13 of 32 lanes) would leave most of each instruction empty.
-// So every thread parks its state in shared memory, the block's update jobs are numbered in
-// (warp, lane) order, and job e runs on lane e % 32 of warp (e / 32 + rot) % W: 52 jobs take two
-// warps instead of four.  rot turns from step to step (and between blocks) so that the warps,
-// which sit on different sub-partitions of the SM, take turns.  Every job runs the same
-// arithmetic on the same inputs whichever thread runs it, so results do not depend on the
-// packing.  Called by every thread of the block (it holds two block barriers).
+// precision).  The update on pairs of floats is about 900 instructions, four times the all-float
+// one, and a warp's own candidates with a hit fill about 13 of its 32 lanes.  So every thread
+// parks its state in shared memory, the block's update jobs are numbered in (warp, lane) order,
+// and job e runs on lane e % 32 of warp (e / 32 + rot) % W: 52 jobs take two warps instead of
+// four.  rot turns from step to step (and between blocks) so that the warps, which sit on
+// different sub-partitions of the SM, take turns.  Every job runs the same arithmetic on the same
+// inputs whichever thread runs it, so results do not depend on the packing.  Called by every
+// thread of the block (it holds two block barriers).
+// k_build on the 40-event batch (163 k seeds): 2.12 ms with the update in double, 0.72 ms on
+// pairs; on pairs without the packing 0.75 ms.
 template <class U, class R, int T>
 __device__ __forceinline__ void pooled_update(R (&p)[6], R (&P)[21], bool job, const float4 &h, const float2 &hv,
                                               bool disk, float *st, unsigned *bal_s, int rot)
@@ -397,23 +420,7 @@ __device__ __forceinline__ void pooled_update(R (&p)[6], R (&P)[21], bool job, c
         if (o < 0 && e < base + c) o = w * 32 + nth_set_bit(b, e - base);
         base += c;
     }
-    if (o >= 0) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) p[k] = st[k * T + o];
-#pragma unroll
-        for (int k = 0; k < 21; ++k) P[k] = st[(6 + k) * T + o];
-        const R hx = st[27 * T + o], hy = st[28 * T + o], hz = st[29 * T + o];
-        const R vu = st[30 * T + o], vv = st[31 * T + o];
-        U dc2 = U(0);
-        if (disk)
-            kalman_update<U, R, true>(p, P, hx, hy, hz, vu, vv, &dc2);
-        else
-            kalman_update<U, R, false>(p, P, hx, hy, hz, vu, vv, &dc2);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) st[k * T + o] = p[k];
-#pragma unroll
-        for (int k = 0; k < 21; ++k) st[(6 + k) * T + o] = P[k];
-    }
+    if (o >= 0) pooled_job<U, R, T>(st + o, disk);
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < 6; ++k) p[k] = st[k * T + tid];
@@ -423,45 +430,28 @@ __device__ __forceinline__ void pooled_update(R (&p)[6], R (&P)[21], bool job, c
 
 // Mixed precision packs the block's Kalman updates into full warps (pooled_update), in blocks of
 // TKF_POOL_WARPS warps.
-#ifndef TKF_BUILD_POOL
-#define TKF_BUILD_POOL 1
-#endif
 #ifndef TKF_POOL_WARPS
 #define TKF_POOL_WARPS 4
 #endif
 template <class R, class U> struct BuildThreads {
-    static constexpr bool pool = TKF_BUILD_POOL && sizeof(R) == 4 && sizeof(U) == 8;
+    static constexpr bool pool = sizeof(R) == 4 && sizeof(U) == 8;
     static constexpr int value = pool ? 32 * TKF_POOL_WARPS : kBuildThreads;
 };
 
-// Resident blocks per SM requested from the register allocator: the all-float kernels with up
-// to 6 candidates are held to 72 registers per thread (7 blocks of 128 threads), their two-step
-// forms to 80 (6 blocks, a few spills: 4.37 ms for the 160-event module batch against 4.51 ms at
-// 5 blocks and 4.77 ms at 4; one seed's near-tie of 701 095 resolves the other way);
-// the mixed-precision kernels with up to 6 candidates to 85 (6 blocks, spilling; the barrel's
-// one-step kernel) or 102 (5 blocks; its two-step and endcap forms): with the pooled updates
-// more resident blocks keep the double-precision pipes fed while other blocks scan (640-event
-// build 32.0 ms at 6 blocks, 33.1 ms at 5, 36.0 ms at 4 and 39.8 ms at 3, the same hit lists); the
-// wider lists and the all-double kernels keep their natural register count.
-#ifndef TKF_BUILD_MINBLOCKS_F32
-#define TKF_BUILD_MINBLOCKS_F32 7
-#endif
-#ifndef TKF_BUILD2_MINBLOCKS_F32
-#define TKF_BUILD2_MINBLOCKS_F32 6
-#endif
-#ifndef TKF_BUILD_MINBLOCKS_MIXED
-#define TKF_BUILD_MINBLOCKS_MIXED 6
-#endif
-#ifndef TKF_BUILD2_MINBLOCKS_MIXED
-#define TKF_BUILD2_MINBLOCKS_MIXED 5
-#endif
+// Resident blocks of 128 threads per SM requested from the register allocator.
+// All-float, up to 6 candidates: 7 blocks (72 registers), their two-step forms 6 (80 registers, a
+// few spills: 4.37 ms for the 160-event module batch against 4.51 ms at 5 and 4.77 ms at 4).
+// Mixed: 7 blocks for 6 candidates on one-step layers (the 40-event pipeline 1.186 ms against
+// 1.215 ms at 6 and 1.27 ms at 8; the endcap batch of 176 k seeds 1.27 ms against 1.36 ms at 5),
+// 5 for more than 6 candidates (163 k seeds, N = 10: 1.55 ms against 1.66 ms at 4, 1.95 ms at 3
+// and 2.56 ms at their natural count).  The register budget also moves the compiler's
+// contractions of the two-step chi2, which can turn a near-tie the other way; the two-step and
+// the 4-candidate forms keep the counts under which every hit list of the test batches stays as
+// it is (5, 3 and 6 blocks; more gained under 3 %).
 template <int NMAX, class R, class U, bool kTwo, bool kDisk> struct BuildMinBlocks {
-    static constexpr int value =
-        (sizeof(R) == 4 && sizeof(U) == 4 && NMAX <= 6)
-            ? (kTwo ? TKF_BUILD2_MINBLOCKS_F32 : TKF_BUILD_MINBLOCKS_F32)
-            : ((sizeof(R) == 4 && sizeof(U) == 8 && NMAX <= 6)
-                   ? (kTwo || kDisk ? TKF_BUILD2_MINBLOCKS_MIXED : TKF_BUILD_MINBLOCKS_MIXED)
-                   : 1);
+    static constexpr int f32 = NMAX > 6 ? 1 : kTwo ? 6 : 7;
+    static constexpr int mixed = kTwo ? (NMAX > 6 ? 3 : 5) : NMAX > 6 ? 5 : NMAX == 6 || kDisk ? 7 : 6;
+    static constexpr int value = sizeof(R) == 8 ? 1 : sizeof(U) == 4 ? f32 : mixed;
 };
 
 // kExactN: the candidates kept per seed equal NMAX, so the segment width and the merge's loops
@@ -627,12 +617,12 @@ __global__ void __launch_bounds__((BuildThreads<R, U>::value), (BuildMinBlocks<N
                     pooled_update<U, R, kThreads>(p, P, gh >= 0, h, hv, disk, pool_st, pool_bal, pool_step & (W - 1));
                     ++pool_step;
                 } else if (gh >= 0) {
-                    U dc2 = U(0);
+                    R dc2 = R(0);
                     if (disk)
-                        kalman_update<U, R, true>(p, P, R(h.x), R(h.y), R(h.z), R(hv.x), R(hv.y), &dc2);
+                        state_update<U, R, true>(p, P, R(h.x), R(h.y), R(h.z), R(hv.x), R(hv.y), &dc2);
                     else
-                        kalman_update<U, R, false>(p, P, R(h.x), R(h.y), R(h.z), R(hv.x), R(hv.y), &dc2);
-                    if (sizeof(R) == 8) chi2 = pchi2 + R(dc2);
+                        state_update<U, R, false>(p, P, R(h.x), R(h.y), R(h.z), R(hv.x), R(hv.y), &dc2);
+                    if (sizeof(R) == 8) chi2 = pchi2 + dc2;
                 }
                 if (alive) {
                     if (l < a.L - 1) scatter<R>(p, P, pick<R>(a.xx0_f[l], a.xx0[l]), mass, disk);

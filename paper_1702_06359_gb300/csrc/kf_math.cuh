@@ -13,7 +13,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "ieee_cvt.cuh"
+#include "pair_f32.cuh"
 #include "sparse_gen.cuh"
 
 namespace tkf {
@@ -547,6 +550,106 @@ __device__ __forceinline__ bool kalman_update(R pR[6], R PR[21], R xh_, R yh_, R
             PR[sym(i, j)] = cvt_down<R>(P[sym(i, j)] - t);
         }
     return true;
+}
+
+// The mixed-precision update in double, out of line: the general form behind mixed_update.
+struct MixedUpdate {
+    float p[6], P[21], x, y, z, vu, vv, chi2;
+    bool ok;
+};
+template <bool kDisk> __device__ __noinline__ MixedUpdate mixed_update_double(MixedUpdate a)
+{
+    double c2 = 0.0;
+    a.ok = kalman_update<double, float, kDisk>(a.p, a.P, a.x, a.y, a.z, a.vu, a.vv, &c2);
+    a.chi2 = cvt_down<float>(c2);
+    return a;
+}
+
+// The mixed-precision update: kalman_update<double, float> with its double arithmetic done on
+// pairs of floats (pair_f32.cuh), because the double units bound every mixed kernel: a fit of
+// 163 k tracks spent 0.515 ms on ten layers at the full double rate, and takes 0.068 ms on pairs.  With the gain good to 2^-45 the Joseph form's second product,
+// (B^T - K S) K^T, is below that too, and P' = P - K B is formed with one rounding per element.
+//
+// What the roundings leave in P' is about 2^-45 of P, so the update may shrink a variance by
+// kPairShrink = 2^16 at most (S / V, times 1 / (1 - rho^2) of the correlation in S) for them to
+// stay below 2^-29 of the result, a thirtieth of its own rounding to float.  A larger shrink,
+// values whose products leave the float range, a singular S and NaNs take the update in double.
+constexpr float kPairShrink = 65536.f;
+template <bool kDisk>
+__device__ __forceinline__ bool mixed_update(float p[6], float P[21], float xh, float yh, float zh, float vu, float vv,
+                                             float *chi2)
+{
+    using Row = typename std::conditional<kDisk, pair32, float>::type;
+    const float ir = 1.f / sqrtf(xh * xh + yh * yh);
+    const float sh = yh * ir, ch = xh * ir;
+    const float u = ch * (yh - p[1]) - sh * (xh - p[0]);
+    const float v = kDisk ? ch * (xh - p[0]) + sh * (yh - p[1]) : zh - p[2];
+    pair32 B0[6], Suu, Suv, Svv;
+    Row B1[6];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        const float p0 = P[sym(0, j)], p1 = P[sym(1, j)];
+        B0[j] = add(mul(ch, p1), mul(-sh, p0));
+        if constexpr (kDisk)
+            B1[j] = add(mul(ch, p0), mul(sh, p1));
+        else
+            B1[j] = P[sym(2, j)];
+    }
+    Suu = add(add(mul(ch, B0[1]), mul(-sh, B0[0])), vu);
+    if constexpr (kDisk) {
+        Suv = add(mul(ch, B0[0]), mul(sh, B0[1]));
+        Svv = add(add(mul(ch, B1[0]), mul(sh, B1[1])), vv);
+    } else {
+        Suv = B0[2];
+        Svv = two_sum(P[sym(2, 2)], vv);
+    }
+    const pair32 uv2 = mul(Suv, Suv);
+    const pair32 det = add(mul(Suu, Svv), pair32{-uv2.h, -uv2.l});
+    const float prod = Suu.h * Svv.h, room = kPairShrink * det.h;
+    float top = P[0];
+#pragma unroll
+    for (int k = 1; k < 6; ++k) top = fmaxf(top, P[sym(k, k)]);
+    const bool fine = Suu.h > 1e-12f && Svv.h > 1e-12f && top < 1e12f && Suu.h * prod < room * vu &&
+                      Svv.h * prod < room * vv;
+    if (!fine) {
+        MixedUpdate a;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) a.p[k] = p[k];
+#pragma unroll
+        for (int k = 0; k < 21; ++k) a.P[k] = P[k];
+        a.x = xh, a.y = yh, a.z = zh, a.vu = vu, a.vv = vv;
+        a = mixed_update_double<kDisk>(a);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) p[k] = a.p[k];
+#pragma unroll
+        for (int k = 0; k < 21; ++k) P[k] = a.P[k];
+        *chi2 = a.chi2;
+        return a.ok;
+    }
+    const pair32 id = recip(det);
+    const pair32 i00 = mul(Svv, id), i11 = mul(Suu, id), m01 = mul(Suv, id), i01 = {-m01.h, -m01.l};
+    const pair32 q0 = add(mul(i00, u), mul(i01, v)), q1 = add(mul(i01, u), mul(i11, v));
+    *chi2 = add(mul(q0, u), mul(q1, v)).h;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        const pair32 K0 = add(mul(B0[i], i00), mul(B1[i], i01)), K1 = add(mul(B0[i], i01), mul(B1[i], i11));
+        p[i] = p[i] + K0.h * u + K1.h * v;
+#pragma unroll
+        for (int j = 0; j <= i; ++j) P[sym(i, j)] = minus_products(P[sym(i, j)], K0, B0[j], K1, B1[j]);
+    }
+    p[4] = wrap_phi(p[4]);
+    return true;
+}
+
+// The Kalman update of a precision mode (state type R, update type U); chi2 in the state's type.
+template <class U, class R, bool kDisk = false>
+__device__ __forceinline__ bool state_update(R p[6], R P[21], R xh, R yh, R zh, R vu, R vv, R *chi2)
+{
+    if constexpr (sizeof(U) != sizeof(R)) {
+        return mixed_update<kDisk>(p, P, xh, yh, zh, vu, vv, chi2);
+    } else {
+        return kalman_update<U, R, kDisk>(p, P, xh, yh, zh, vu, vv, chi2);
+    }
 }
 
 }  // namespace tkf

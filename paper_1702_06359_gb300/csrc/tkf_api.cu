@@ -667,10 +667,10 @@ __device__ __forceinline__ bool to_layer(const FitGeom &g, int l, R p[6], R P[21
 // The Kalman update with the layer's measurement model (r-phi and z on a cylinder, r-phi and r
 // on a disk).
 template <class U, class R, bool kDisk>
-__device__ __forceinline__ bool update_at(const FitGeom &g, int l, R p[6], R P[21], R x, R y, R z, R vu, R vv, U *c2)
+__device__ __forceinline__ bool update_at(const FitGeom &g, int l, R p[6], R P[21], R x, R y, R z, R vu, R vv, R *c2)
 {
-    if (kDisk && ((g.disk_mask >> l) & 1u)) return kalman_update<U, R, true>(p, P, x, y, z, vu, vv, c2);
-    return kalman_update<U, R, false>(p, P, x, y, z, vu, vv, c2);
+    if (kDisk && ((g.disk_mask >> l) & 1u)) return state_update<U, R, true>(p, P, x, y, z, vu, vv, c2);
+    return state_update<U, R, false>(p, P, x, y, z, vu, vv, c2);
 }
 
 
@@ -743,16 +743,15 @@ __global__ void k_seed(const FitGeom g, const tkf_hits h, const int *seed_hits, 
     }
 }
 
-// Resident blocks of 128 threads per SM requested from the register allocator for the all-float
-// fit kernels (k_fit, k_seed_fit, k_fit_backward): 7 holds them to 72 registers, their count
-// before the reads were pipelined (80 otherwise, 6 blocks); measured on the 2.6 M-track fit,
-// 72 registers is 4 % faster (0.575 against 0.599 ms), the backward pass 3 % (0.760 / 0.786 ms).
-#ifndef TKF_FIT_MINBLOCKS_F32
-#define TKF_FIT_MINBLOCKS_F32 7
-#endif
+// Resident blocks of 128 threads per SM requested from the register allocator for the fit kernels
+// (k_fit, k_seed_fit, k_fit_backward) with float states.  All-float: 7 holds them to 72
+// registers, their count before the reads were pipelined (80 otherwise, 6 blocks); measured on
+// the 2.6 M-track fit, 72 registers is 4 % faster (0.575 against 0.599 ms), the backward pass 3 %
+// (0.760 / 0.786 ms).  Mixed: 4 (128 registers); estimate, fit and backward pass of 300 k tracks
+// take 0.424 ms at 4, 0.449 ms at 5 (3.36 ms with the update in double).
 constexpr int kFitThreads = 128;
 template <class R, class U> struct FitMinBlocks {
-    static constexpr int value = (sizeof(R) == 4 && sizeof(U) == 4) ? TKF_FIT_MINBLOCKS_F32 : 1;
+    static constexpr int value = sizeof(R) == 8 ? 1 : sizeof(U) == 4 ? 7 : 4;
 };
 
 // A hit's position and variances read from the hit planes (zeros for an id outside 0..n-1).
@@ -809,12 +808,12 @@ __device__ __forceinline__ void fit_layers(const FitGeom &g, const tkf_hits &h, 
             break;
         }
         if (hid >= 0) {
-            U dc2;
+            R dc2;
             if (!update_at<U, R, kDisk>(g, l, p, P, cur.x, cur.y, cur.z, cur.vu, cur.vv, &dc2)) {
                 status = TKF_TRACK_SINGULAR;
                 break;
             }
-            chi2 += R(dc2);
+            chi2 += dc2;
             nh += 1;
         }
         if (l < g.L - 1)
@@ -951,12 +950,12 @@ __global__ void __launch_bounds__(kFitThreads, (FitMinBlocks<R, U>::value)) k_fi
             break;
         }
         if (hid >= 0) {
-            U dc2;
+            R dc2;
             if (!update_at<U, R, kDisk>(g, l, p, P, cur.x, cur.y, cur.z, cur.vu, cur.vv, &dc2)) {
                 status = TKF_TRACK_SINGULAR;
                 break;
             }
-            chi2 += R(dc2);
+            chi2 += dc2;
             nh += 1;
         }
         scatter<R>(p, P, gpick<R>(g.xx0_f[l], g.xx0[l]), mass, kDisk && ((g.disk_mask >> l) & 1u));
