@@ -443,22 +443,25 @@ template <class R, class U> struct BuildThreads {
 // few spills: 4.37 ms for the 160-event module batch against 4.51 ms at 5 and 4.77 ms at 4).
 // Mixed: 7 blocks for 6 candidates on one-step layers (the 40-event pipeline 1.186 ms against
 // 1.215 ms at 6 and 1.27 ms at 8; the endcap batch of 176 k seeds 1.27 ms against 1.36 ms at 5),
-// 5 for more than 6 candidates (163 k seeds, N = 10: 1.55 ms against 1.66 ms at 4, 1.95 ms at 3
+// 5 for 10 candidates (163 k seeds: 1.55 ms against 1.66 ms at 4, 1.95 ms at 3
 // and 2.56 ms at their natural count).  The register budget also moves the compiler's
 // contractions of the two-step chi2, which can turn a near-tie the other way; the two-step and
 // the 4-candidate forms keep the counts under which every hit list of the test batches stays as
 // it is (5, 3 and 6 blocks; more gained under 3 %).
-template <int NMAX, class R, class U, bool kTwo, bool kDisk> struct BuildMinBlocks {
-    static constexpr int f32 = NMAX > 6 ? 1 : kTwo ? 6 : 7;
-    static constexpr int mixed = kTwo ? (NMAX > 6 ? 3 : 5) : NMAX > 6 ? 5 : NMAX == 6 || kDisk ? 7 : 6;
-    static constexpr int value = sizeof(R) == 8 ? 1 : sizeof(U) == 4 ? f32 : mixed;
+// All-float, N = 10: 6 blocks one-step (183 k seeds 1.40 ms against 1.68 ms at their natural 112
+// registers; endcaps 1.23 against 1.47 ms), 5 where N < 10 runs on the 10-entry lists (0.86
+// against 0.95 ms), 4 two-step (3.29 against 3.78 ms), again without a changed hit list.
+template <int NMAX, class R, class U, bool kTwo, bool kExactN, bool kDisk> struct BuildMinBlocks {
+    static constexpr int f32 = NMAX == 10 ? (kTwo ? 4 : kExactN ? 6 : 5) : kTwo ? 6 : 7;
+    static constexpr int mixed = NMAX == 10 ? (kTwo ? 3 : 5) : kTwo ? 5 : NMAX == 6 || kDisk ? 7 : 6;
+    static constexpr int value = sizeof(R) == 8 || NMAX > 10 ? 1 : sizeof(U) == 4 ? f32 : mixed;
 };
 
 // kExactN: the candidates kept per seed equal NMAX, so the segment width and the merge's loops
 // are compile-time constants (unrolled); otherwise N = a.ncand <= NMAX at run time.
 // kDisk: the configuration has endcap disks; each layer then goes by its kind (cylinder or disk).
 template <int NMAX, class R, class U, bool kTwo, bool kExactN, bool kDisk>
-__global__ void __launch_bounds__((BuildThreads<R, U>::value), (BuildMinBlocks<NMAX, R, U, kTwo, kDisk>::value))
+__global__ void __launch_bounds__((BuildThreads<R, U>::value), (BuildMinBlocks<NMAX, R, U, kTwo, kExactN, kDisk>::value))
     k_build(const BuildArgs a)
 {
     constexpr int kThreads = BuildThreads<R, U>::value;
