@@ -99,6 +99,9 @@ int seed_order_reserve(tkf_ctx *ctx, size_t max_seeds, size_t max_events);
 // pipeline).
 int first_list_reserve(tkf_ctx *ctx, size_t max_seeds);
 
+// Frees the seeding scratch of a context.
+void seed_scratch_free(tkf_ctx *ctx);
+
 inline int build_nmax(int n)
 {
     return n <= 1 ? 1 : n <= 4 ? 4 : n <= 6 ? 6 : n <= 10 ? 10 : 16;
@@ -121,10 +124,14 @@ struct tkf_ctx {
     unsigned *first_key = nullptr;
     int *first_hit = nullptr;
     size_t first_cap = 0;
-    // seeding scratch: best layer-1 / layer-2 hit and score per sorted hit position, seeds per block
-    int *seed_b = nullptr, *seed_c = nullptr, *seed_cnt = nullptr;
+    // seeding scratch: best layer-1 / layer-2 hit and score per first hit, first hits before each
+    // event, the grids of layers 2 and 3 (SeedCells, cell tables, hits in cell order), seeds per
+    // compaction block and the tile queue
+    int *seed_b = nullptr, *seed_c = nullptr, *seed_first = nullptr, *seed_tab = nullptr, *seed_id = nullptr,
+        *seed_cnt = nullptr;
     float *seed_s = nullptr;
-    size_t seed_cap = 0, seed_cnt_cap = 0;
+    void *seed_cells = nullptr, *seed_xyzr = nullptr;
+    size_t seed_cap = 0, seed_cap_events = 0, seed_cap_tab = 0;
 };
 
 struct tkf_hit_index {
