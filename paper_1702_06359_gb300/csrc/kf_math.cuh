@@ -81,6 +81,65 @@ __host__ __device__ __forceinline__ float fast_div(float a, float b)
 }
 __host__ __device__ __forceinline__ double fast_div(double a, double b) { return a / b; }
 
+// ------------------------------------------------------------------ float <-> double without the FP64 unit
+// (ieee_cvt.cuh): the mixed-precision update converts with integer operations on the bit fields.
+#ifndef TKF_INT_CVT
+#define TKF_INT_CVT 1
+#endif
+
+// cvt_up<U>(x): x (float or double) as U; cvt_down<R>(x): x (double) as R (float or double).
+template <class U> __device__ __forceinline__ U cvt_up(float x)
+{
+#if TKF_INT_CVT
+    if constexpr (sizeof(U) == 8) return f32_to_f64_bits(x);
+#endif
+    return U(x);
+}
+template <class U> __device__ __forceinline__ U cvt_up(double x) { return U(x); }
+template <class R> __device__ __forceinline__ R cvt_down(float x) { return R(x); }
+template <class R> __device__ __forceinline__ R cvt_down(double x)
+{
+#if TKF_INT_CVT
+    if constexpr (sizeof(R) == 4) return f64_to_f32_bits(x);
+#endif
+    return R(x);
+}
+
+// 1/x: in float the approximate division; in double Newton's iteration for the
+// reciprocal, y <- y (2 - x y) written as y + y (1 - x y), from the correctly rounded
+// single-precision reciprocal of x rounded to float (relative error below 2^-23; each step
+// squares it, so two steps reach double rounding) -- four double operations where the IEEE
+// division takes about three times as many on the scarce double-precision units.  An x outside
+// the float range takes the IEEE division.
+template <class U> __device__ __forceinline__ U recip(U x) { return U(1) / x; }
+template <> __device__ __forceinline__ double recip<double>(double x)
+{
+#if TKF_INT_CVT
+    const float xf = f64_to_f32_bits(x);
+    const float yf = __frcp_rn(xf);
+    if (!(fabsf(xf) > 1e-37f && fabsf(xf) < 1e37f)) return 1.0 / x;
+    double y = f32_to_f64_bits(yf);
+    y = fma(y, fma(-x, y, 1.0), y);
+    y = fma(y, fma(-x, y, 1.0), y);
+    return y;
+#else
+    return 1.0 / x;
+#endif
+}
+
+// 1/sqrt(x): Newton's iteration for the inverse square root, y <- y + y (1 - x y^2) / 2, twice from
+// the single-precision one (relative error 2^-22; each step squares it, times 3/2).
+template <class R> __device__ __forceinline__ R inv_sqrt(R x) { return R(1) / sq(x); }
+template <> __device__ __forceinline__ double inv_sqrt<double>(double x)
+{
+    const float xf = f64_to_f32_bits(x);
+    if (!(xf > 1e-37f && xf < 1e37f)) return 1.0 / sqrt(x);
+    double y = f32_to_f64_bits(rsqrtf(xf));
+    y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+    y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+    return y;
+}
+
 template <class R> struct Lim;
 template <> struct Lim<float> {
     static constexpr float series = 0.25f;  // |kappa s| below which the helix functions use series
@@ -92,7 +151,10 @@ template <> struct Lim<float> {
     static constexpr float converged = 1e-6f;
 };
 template <> struct Lim<double> {
-    static constexpr double series = 0.05;
+    // with two terms more than float's series below: within 2^-53 up to here, so that a warp's tracks
+    // above 0.2 GeV between layers 4 cm apart all take the series (sincos of some lanes and the series
+    // of the others both ran before)
+    static constexpr double series = 0.25;
     static constexpr int newton = 4;
     static constexpr double converged = 1e-13;
 };
@@ -111,10 +173,15 @@ template <class R> __host__ __device__ __forceinline__ void helix_fn(R a, R &S, 
 {
     if (ab(a) < Lim<R>::series) {
         const R a2 = a * a;
-        S = R(1) + a2 * (R(-1.0 / 6) + a2 * (R(1.0 / 120) + a2 * (R(-1.0 / 5040) + a2 * R(1.0 / 362880))));
-        C = a * (R(0.5) + a2 * (R(-1.0 / 24) + a2 * (R(1.0 / 720) + a2 * (R(-1.0 / 40320) + a2 * R(1.0 / 3628800)))));
-        Sd = a * (R(-1.0 / 3) + a2 * (R(1.0 / 30) + a2 * (R(-1.0 / 840) + a2 * (R(1.0 / 45360) - a2 * R(1.0 / 3991680)))));
-        Cd = R(0.5) + a2 * (R(-1.0 / 8) + a2 * (R(1.0 / 144) + a2 * (R(-1.0 / 5760) + a2 * R(1.0 / 403200))));
+        // the series' ends: one term more in double
+        const R s9 = sizeof(R) == 8 ? R(1.0 / 362880) - a2 * R(1.0 / 39916800) : R(1.0 / 362880);
+        const R c9 = sizeof(R) == 8 ? R(1.0 / 3628800) - a2 * R(1.0 / 479001600) : R(1.0 / 3628800);
+        const R t9 = sizeof(R) == 8 ? R(1.0 / 3991680) - a2 * R(1.0 / 518918400) : R(1.0 / 3991680);
+        const R d9 = sizeof(R) == 8 ? R(1.0 / 403200) - a2 * R(1.0 / 43545600) : R(1.0 / 403200);
+        S = R(1) + a2 * (R(-1.0 / 6) + a2 * (R(1.0 / 120) + a2 * (R(-1.0 / 5040) + a2 * s9)));
+        C = a * (R(0.5) + a2 * (R(-1.0 / 24) + a2 * (R(1.0 / 720) + a2 * (R(-1.0 / 40320) + a2 * c9))));
+        Sd = a * (R(-1.0 / 3) + a2 * (R(1.0 / 30) + a2 * (R(-1.0 / 840) + a2 * (R(1.0 / 45360) - a2 * t9))));
+        Cd = R(0.5) + a2 * (R(-1.0 / 8) + a2 * (R(1.0 / 144) + a2 * (R(-1.0 / 5760) + a2 * d9)));
     } else {
         R sn, cs;
         sc(a, &sn, &cs);
@@ -124,6 +191,18 @@ template <class R> __host__ __device__ __forceinline__ void helix_fn(R a, R &S, 
         Sd = (cs - S) * ia;
         Cd = (sn - C) * ia;
     }
+}
+
+// sin and cos of a state's phi and theta
+template <class R> struct Trig {
+    R sp, cp, st, ct;
+};
+template <class R> __device__ __forceinline__ Trig<R> trig_of(const R p[6])
+{
+    Trig<R> t;
+    sc(p[4], &t.sp, &t.cp);
+    sc(p[5], &t.st, &t.ct);
+    return t;
 }
 
 // ------------------------------------------------------------------ propagation (Sec. 2.2)
@@ -151,9 +230,136 @@ template <class R> __host__ __device__ __forceinline__ void helix_fn(R a, R &S, 
 //     (radius^2 - r0^2) / (A + sqrt(disc)).
 enum : int { kPropOut = 0, kPropIn = 1, kPropStep = 2 };
 
-template <class R, int kMode = kPropOut>
-__host__ __device__ __forceinline__ bool propagate(R p[6], R P[21], R radius, R kb)
+// The start of an inward step whose tangent line misses the cylinder: the nearer crossing ahead of
+// the track circle and the cylinder (see propagate).
+template <class R>
+__device__ __forceinline__ bool circle_crossing(R x, R y, R sp, R cp, R kappa, R radius, R &s)
 {
+    if (!(ab(kappa) > R(0))) return false;
+    const R ik = R(1) / kappa;
+    const R cx = x - sp * ik, cy = y + cp * ik;  // centre of the track circle
+    const R d2 = cx * cx + cy * cy, d = sq(d2);
+    const R a = (radius * radius - ik * ik + d2) / (R(2) * d);  // chord's distance from the origin
+    const R h2 = radius * radius - a * a;
+    if (!(h2 >= R(0)) || !(d > R(0))) return false;
+    const R h = sq(h2);
+    const R ux = x - cx, uy = y - cy;  // p0 - c
+    const R two_pi_rho = R(2.0 * kPi) * ab(ik);
+    s = R(-1);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const R sg = k ? R(-1) : R(1);
+        const R qx = (a * cx - sg * h * cy) / d - cx, qy = (a * cy + sg * h * cx) / d - cy;  // crossing - c
+        R sk = at2(ux * qy - uy * qx, ux * qx + uy * qy) * ik;
+        if (!(sk > R(0))) sk += two_pi_rho;
+        if (s < R(0) || sk < s) s = sk;
+    }
+    return true;
+}
+
+// The double form.  What bounds the double kernels is the double pipe (one warp instruction in 64
+// cycles), so everything that double rounding does not need is done in float: the first two Newton
+// steps (the first two of float's own count bring s within about 1e-5 cm; the two double steps that
+// follow square that twice) and the reciprocals of the double steps' derivatives.  Divisions are
+// Newton reciprocals.  A start that is neither outward nor clear of the tangent takes every step in
+// double, as far as the float form's rule says.
+template <int kMode>
+__device__ __forceinline__ bool propagate_f64(double p[6], double P[21], double radius, double kb, const Trig<double> &t)
+{
+    const double x = p[0], y = p[1], z = p[2], w = p[3], phi = p[4];
+    const double sp = t.sp, cp = t.cp;
+    const double kappa = -kb * w;
+    const double A = x * cp + y * sp;
+    const double q = radius * radius - (x * x + y * y);
+    const double disc = A * A + q;
+    if (kMode == kPropStep && !(A > 0.0)) return false;
+    if (kMode != kPropIn && !(disc >= 0.0)) return false;
+    const bool clear = kMode != kPropIn || disc > 0.01 * radius * radius;
+    double S, C, Sd, Cd, s;
+    float sf = INFINITY;
+    if (clear) {
+        const float xf = cvt_down<float>(x), yf = cvt_down<float>(y), spf = cvt_down<float>(sp),
+                    cpf = cvt_down<float>(cp), kf = cvt_down<float>(kappa), Af = cvt_down<float>(A),
+                    Rf = cvt_down<float>(radius), df = sqrtf(cvt_down<float>(disc));
+        sf = kMode == kPropStep ? cvt_down<float>(q) / (Af + df) : (kMode == kPropOut ? -Af + df : -Af - df);
+#pragma unroll
+        for (int it = 0; it < 2; ++it) {
+            float Sf, Cf, Sdf, Cdf;
+            const float a = kf * sf;
+            helix_fn(a, Sf, Cf, Sdf, Cdf);
+            const float sa = a * Sf, ca = 1.f - a * Cf;
+            const float xs = xf + sf * (cpf * Sf - spf * Cf), ys = yf + sf * (spf * Sf + cpf * Cf);
+            sf -= (xs * xs + ys * ys - Rf * Rf) / (2.f * (xs * (cpf * ca - spf * sa) + ys * (spf * ca + cpf * sa)));
+        }
+    }
+    if (fabsf(sf) < 1e30f) {
+        s = cvt_up<double>(sf);
+#pragma unroll
+        for (int it = 0; it < 2; ++it) {
+            const double a = kappa * s;
+            helix_fn(a, S, C, Sd, Cd);
+            const double sa = a * S, ca = 1.0 - a * C;
+            const double xs = x + s * (cp * S - sp * C), ys = y + s * (sp * S + cp * C);
+            const double g = xs * xs + ys * ys - radius * radius;
+            const double dg = xs * (cp * ca - sp * sa) + ys * (sp * ca + cp * sa);
+            s -= g * cvt_up<double>(0.5f / cvt_down<float>(dg));
+        }
+    } else {
+        if (kMode == kPropStep) {
+            s = q / (A + sqrt(disc));
+        } else if (kMode == kPropOut) {
+            s = -A + sqrt(disc);
+        } else if (disc >= 0.0) {
+            s = -A - sqrt(disc);
+        } else if (!circle_crossing<double>(x, y, sp, cp, kappa, radius, s)) {
+            return false;
+        }
+        constexpr int n_newton = kMode == kPropIn ? 3 * Lim<double>::newton + 2 : Lim<double>::newton;
+        for (int it = 0; it < n_newton; ++it) {
+            const double a = kappa * s;
+            helix_fn(a, S, C, Sd, Cd);
+            const double sa = a * S, ca = 1.0 - a * C;
+            const double xs = x + s * (cp * S - sp * C), ys = y + s * (sp * S + cp * C);
+            const double g = xs * xs + ys * ys - radius * radius;
+            const double ds = g / (2.0 * (xs * (cp * ca - sp * sa) + ys * (sp * ca + cp * sa)));
+            s -= ds;
+            if (kMode == kPropIn && it + 1 >= Lim<double>::newton && (clear || ab(ds) <= Lim<double>::converged * ab(s)))
+                break;
+        }
+    }
+    const double a = kappa * s;
+    helix_fn(a, S, C, Sd, Cd);
+    const double sa = a * S, ca = 1.0 - a * C;
+    const double xs = x + s * (cp * S - sp * C), ys = y + s * (sp * S + cp * C);
+    const double c1 = cp * ca - sp * sa, s1 = sp * ca + cp * sa;
+    const double D = xs * c1 + ys * s1;  // r dr/ds
+    if (kMode == kPropStep ? !(D > 1e-6 * radius) : (!(s > 0.0) || !(ab(D) > 1e-6 * radius))) return false;
+    if (!(ab(xs * xs + ys * ys - radius * radius) < 1e-3 * radius)) return false;
+    const double ist = recip(t.st), cot = t.ct * ist;
+    // the Jacobian as in propagate
+    const double s2kb = -kb * s * s;
+    const double dx_dw = s2kb * (cp * Sd - sp * Cd), dy_dw = s2kb * (sp * Sd + cp * Cd);
+    const double dx_dphi = -(ys - y), dy_dphi = xs - x;
+    const double iD = recip(D);
+    const double s_x = -xs * iD, s_y = -ys * iD;
+    const double s_w = -(xs * dx_dw + ys * dy_dw) * iD, s_f = -(xs * dx_dphi + ys * dy_dphi) * iD;
+    double Q[21];
+    transport_cov<double>(1.0 + c1 * s_x, c1 * s_y, dx_dw + c1 * s_w, dx_dphi + c1 * s_f, s1 * s_x, 1.0 + s1 * s_y,
+                          dy_dw + s1 * s_w, dy_dphi + s1 * s_f, cot * s_x, cot * s_y, cot * s_w, cot * s_f,
+                          -s * ist * ist, kappa * s_x, kappa * s_y, -kb * s + kappa * s_w, 1.0 + kappa * s_f, P, Q);
+#pragma unroll
+    for (int k = 0; k < 21; ++k) P[k] = Q[k];
+    p[0] = xs;
+    p[1] = ys;
+    p[2] = z + s * cot;
+    p[4] = wrap_phi(phi + a);
+    return true;
+}
+
+template <class R, int kMode = kPropOut>
+__device__ __forceinline__ bool propagate(R p[6], R P[21], R radius, R kb)
+{
+    if constexpr (sizeof(R) == 8) return propagate_f64<kMode>(p, P, radius, kb, trig_of(p));
     const R x = p[0], y = p[1], z = p[2], w = p[3], phi = p[4], th = p[5];
     R sp, cp;
     sc(phi, &sp, &cp);
@@ -171,25 +377,7 @@ __host__ __device__ __forceinline__ bool propagate(R p[6], R P[21], R radius, R 
     } else if (disc >= R(0)) {
         s = -A - sq(disc);
     } else {
-        if (!(ab(kappa) > R(0))) return false;
-        const R ik = R(1) / kappa;
-        const R cx = x - sp * ik, cy = y + cp * ik;  // centre of the track circle
-        const R d2 = cx * cx + cy * cy, d = sq(d2);
-        const R a = (radius * radius - ik * ik + d2) / (R(2) * d);  // chord's distance from the origin
-        const R h2 = radius * radius - a * a;
-        if (!(h2 >= R(0)) || !(d > R(0))) return false;
-        const R h = sq(h2);
-        const R ux = x - cx, uy = y - cy;  // p0 - c
-        const R two_pi_rho = R(2.0 * kPi) * ab(ik);
-        s = R(-1);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const R sg = k ? R(-1) : R(1);
-            const R qx = (a * cx - sg * h * cy) / d - cx, qy = (a * cy + sg * h * cx) / d - cy;  // crossing - c
-            R sk = at2(ux * qy - uy * qx, ux * qx + uy * qy) * ik;
-            if (!(sk > R(0))) sk += two_pi_rho;
-            if (s < R(0) || sk < s) s = sk;
-        }
+        if (!circle_crossing<R>(x, y, sp, cp, kappa, radius, s)) return false;
     }
     R S, C, Sd, Cd;
     // inward starts can be far from the crossing (a grazing entry, the circle intersection's
@@ -260,8 +448,39 @@ __host__ __device__ __forceinline__ bool propagate(R p[6], R P[21], R radius, R 
 // ds/dz = -1/cot(theta) and ds/dtheta = s / (sin^2(theta) cot(theta)) from z(s, p_in) = zp (the
 // path does not depend on x, y, q/pT, phi); P <- J P J^T from that sparsity (plane_cov).
 // Returns false when the plane is behind, parallel, or more than a full turn away (a looper).
-template <class R> __host__ __device__ __forceinline__ bool propagate_plane(R p[6], R P[21], R zp, R kb)
+__device__ __forceinline__ bool propagate_plane_f64(double p[6], double P[21], double zp, double kb,
+                                                    const Trig<double> &t)
 {
+    const double x = p[0], y = p[1], phi = p[4];
+    const double ist = recip(t.st), cot = t.ct * ist;
+    if (!(ab(cot) > 0.0)) return false;
+    const double icot = recip(cot), s = (zp - p[2]) * icot;
+    const double kappa = -kb * p[3];
+    if (!(s > 0.0) || !(ab(kappa) * s <= 2.0 * kPi)) return false;
+    const double sp = t.sp, cp = t.cp;
+    const double a = kappa * s;
+    double S, C, Sd, Cd;
+    helix_fn(a, S, C, Sd, Cd);
+    const double sa = a * S, ca = 1.0 - a * C;
+    const double xs = x + s * (cp * S - sp * C), ys = y + s * (sp * S + cp * C);
+    const double c1 = cp * ca - sp * sa, s1 = sp * ca + cp * sa;
+    const double s2kb = -kb * s * s;
+    const double sth = s * ist * ist * icot;
+    double Q[21];
+    plane_cov<double>(-c1 * icot, s2kb * (cp * Sd - sp * Cd), -(ys - y), c1 * sth, -s1 * icot, s2kb * (sp * Sd + cp * Cd),
+                      xs - x, s1 * sth, -kappa * icot, -kb * s, kappa * sth, P, Q);
+#pragma unroll
+    for (int k = 0; k < 21; ++k) P[k] = Q[k];
+    p[0] = xs;
+    p[1] = ys;
+    p[2] = zp;
+    p[4] = wrap_phi(phi + a);
+    return true;
+}
+
+template <class R> __device__ __forceinline__ bool propagate_plane(R p[6], R P[21], R zp, R kb)
+{
+    if constexpr (sizeof(R) == 8) return propagate_plane_f64(p, P, zp, kb, trig_of(p));
     const R x = p[0], y = p[1], z = p[2], w = p[3], phi = p[4], th = p[5];
     R st, ct;
     sc(th, &st, &ct);
@@ -301,9 +520,32 @@ template <class R> __host__ __device__ __forceinline__ bool propagate_plane(R p[
 // two kicks orthogonal to the direction add theta0^2 to theta, theta0^2/sin^2(theta) to phi,
 // and (through pT = p sin(theta) at fixed p) the q/pT terms.
 // disk: the layer is an endcap disk, whose normal is the z axis (|cos alpha| = |cos theta|).
-template <class R>
-__host__ __device__ __forceinline__ void scatter(const R p[6], R P[21], R xx0, R mass, bool disk = false)
+// The double form: v in terms of 1 / p^2 = w^2 sin^2(theta) and 1 / beta^2 = 1 + m^2 / p^2, without the
+// square roots that v squares away, and with Newton reciprocals.
+__device__ __forceinline__ void scatter_f64(const double p[6], double P[21], double xx0, double mass, bool disk,
+                                            const Trig<double> &t)
 {
+    if (!(xx0 > 0.0)) return;
+    const double w = p[3], ist = recip(t.st), cot = t.ct * ist;
+    const double ip2 = (w * t.st) * (w * t.st), ib2 = 1.0 + mass * mass * ip2;
+    const double cosa = disk ? ab(t.ct)
+                             : ab(t.st * (p[0] * t.cp + p[1] * t.sp)) * inv_sqrt(p[0] * p[0] + p[1] * p[1]);
+    const double th = xx0 * recip(cosa);
+    const double f = 0.0136 * (1.0 + 0.038 * log(th * ib2));
+    const double v = f * f * th * ib2 * ip2, wc = w * cot;
+    P[sym(3, 3)] += wc * wc * v;
+    P[sym(5, 3)] += -wc * v;
+    P[sym(4, 4)] += v * (ist * ist);
+    P[sym(5, 5)] += v;
+}
+
+template <class R>
+__device__ __forceinline__ void scatter(const R p[6], R P[21], R xx0, R mass, bool disk = false)
+{
+    if constexpr (sizeof(R) == 8) {
+        scatter_f64(p, P, xx0, mass, disk, trig_of(p));
+        return;
+    }
     if (!(xx0 > R(0))) return;
     R st, ct, sp, cp;
     fast_sc(p[5], &st, &ct);
@@ -445,52 +687,6 @@ __host__ __device__ __forceinline__ R step_chi2(const R p[6], const R P[21], R s
     return fast_div(u * (Svv * u - R(2) * Suv * v) + Suu * v * v, det);
 }
 
-// ------------------------------------------------------------------ float <-> double without the FP64 unit
-// (ieee_cvt.cuh): the mixed-precision update converts with integer operations on the bit fields.
-#ifndef TKF_INT_CVT
-#define TKF_INT_CVT 1
-#endif
-
-// cvt_up<U>(x): x (float or double) as U; cvt_down<R>(x): x (double) as R (float or double).
-template <class U> __device__ __forceinline__ U cvt_up(float x)
-{
-#if TKF_INT_CVT
-    if constexpr (sizeof(U) == 8) return f32_to_f64_bits(x);
-#endif
-    return U(x);
-}
-template <class U> __device__ __forceinline__ U cvt_up(double x) { return U(x); }
-template <class R> __device__ __forceinline__ R cvt_down(float x) { return R(x); }
-template <class R> __device__ __forceinline__ R cvt_down(double x)
-{
-#if TKF_INT_CVT
-    if constexpr (sizeof(R) == 4) return f64_to_f32_bits(x);
-#endif
-    return R(x);
-}
-
-// 1/x for x > 0: in float the approximate division; in double Newton's iteration for the
-// reciprocal, y <- y (2 - x y) written as y + y (1 - x y), from the correctly rounded
-// single-precision reciprocal of x rounded to float (relative error below 2^-23; each step
-// squares it, so two steps reach double rounding) -- four double operations where the IEEE
-// division takes about three times as many on the scarce double-precision units.  An x outside
-// the float range takes the IEEE division.
-template <class U> __device__ __forceinline__ U recip(U x) { return U(1) / x; }
-template <> __device__ __forceinline__ double recip<double>(double x)
-{
-#if TKF_INT_CVT
-    const float xf = f64_to_f32_bits(x);
-    const float yf = __frcp_rn(xf);
-    if (!(xf > 1e-37f && xf < 1e37f)) return 1.0 / x;
-    double y = f32_to_f64_bits(yf);
-    y = fma(y, fma(-x, y, 1.0), y);
-    y = fma(y, fma(-x, y, 1.0), y);
-    return y;
-#else
-    return 1.0 / x;
-#endif
-}
-
 // Kalman update with the Joseph-form covariance:
 //   B = H P (2x6), S = B H^T + V, K = B^T S^-1, p += K r,
 //   P' = (I - K H) P (I - K H)^T + K V K^T = P - K B - (B^T - K S) K^T   (element-wise below).
@@ -503,7 +699,7 @@ template <> __device__ __forceinline__ double recip<double>(double x)
 template <class U, class R, bool kDisk = false>
 __device__ __forceinline__ bool kalman_update(R pR[6], R PR[21], R xh_, R yh_, R zh_, R vu_, R vv_, U *chi2)
 {
-    const R irR = R(1) / sq(xh_ * xh_ + yh_ * yh_);
+    const R irR = inv_sqrt(xh_ * xh_ + yh_ * yh_);
     const R shR = yh_ * irR, chR = xh_ * irR;
     const R uR = chR * (yh_ - pR[1]) - shR * (xh_ - pR[0]);
     const R vR = kDisk ? chR * (xh_ - pR[0]) + shR * (yh_ - pR[1]) : zh_ - pR[2];
@@ -543,11 +739,18 @@ __device__ __forceinline__ bool kalman_update(R pR[6], R PR[21], R xh_, R yh_, R
     for (int i = 0; i < 6; ++i)
 #pragma unroll
         for (int j = 0; j <= i; ++j) {
-            U t = K0[i] * B0[j];
-            t = fma(K1[i], B1[j], t);
-            t = fma(D0[i], K0[j], t);
-            t = fma(D1[i], K1[j], t);
-            PR[sym(i, j)] = cvt_down<R>(P[sym(i, j)] - t);
+            if constexpr (sizeof(U) == 8) {  // one operation fewer on the double pipe
+                U t = fma(-K0[i], B0[j], P[sym(i, j)]);
+                t = fma(-K1[i], B1[j], t);
+                t = fma(-D0[i], K0[j], t);
+                PR[sym(i, j)] = cvt_down<R>(fma(-D1[i], K1[j], t));
+            } else {
+                U t = K0[i] * B0[j];
+                t = fma(K1[i], B1[j], t);
+                t = fma(D0[i], K0[j], t);
+                t = fma(D1[i], K1[j], t);
+                PR[sym(i, j)] = cvt_down<R>(P[sym(i, j)] - t);
+            }
         }
     return true;
 }

@@ -655,13 +655,29 @@ struct FitGeom {
 // The state's move to layer l (kDisk: the kernel serves configurations with endcap disks):
 // the layer's cylinder (at target_radius), or the disk on the side of the state's z.
 template <class R, bool kDisk, int kMode = kPropOut>
-__device__ __forceinline__ bool to_layer(const FitGeom &g, int l, R p[6], R P[21], R radius, R kb)
+__device__ __forceinline__ bool to_layer(const FitGeom &g, int l, R p[6], R P[21], R radius, R kb, const Trig<R> &t)
 {
     if (kDisk && ((g.disk_mask >> l) & 1u)) {
-        const R zd = gpick<R>(g.disk_z_f[l], g.disk_z[l]);
-        return propagate_plane<R>(p, P, p[2] >= R(0) ? zd : -zd, kb);
+        const R zd = gpick<R>(g.disk_z_f[l], g.disk_z[l]), zp = p[2] >= R(0) ? zd : -zd;
+        if constexpr (sizeof(R) == 8) return propagate_plane_f64(p, P, zp, kb, t);
+        return propagate_plane<R>(p, P, zp, kb);
     }
+    if constexpr (sizeof(R) == 8) return propagate_f64<kMode>(p, P, radius, kb, t);
     return propagate<R, kMode>(p, P, radius, kb);
+}
+
+// The material of layer l.  In double the angles' sines and cosines (t) are formed once per layer,
+// for the scattering and the step that follows it; the float forms use their own, faster ones.
+template <class R>
+__device__ __forceinline__ void scatter_at(const FitGeom &g, int l, R p[6], R P[21], R mass, bool disk, Trig<R> &t)
+{
+    const R xx0 = gpick<R>(g.xx0_f[l], g.xx0[l]);
+    if constexpr (sizeof(R) == 8) {
+        t = trig_of(p);
+        scatter_f64(p, P, xx0, mass, disk, t);
+    } else {
+        scatter<R>(p, P, xx0, mass, disk);
+    }
 }
 
 // The Kalman update with the layer's measurement model (r-phi and z on a cylinder, r-phi and r
@@ -749,7 +765,11 @@ __global__ void k_seed(const FitGeom g, const tkf_hits h, const int *seed_hits, 
 // the 2.6 M-track fit, 72 registers is 4 % faster (0.575 against 0.599 ms), the backward pass 3 %
 // (0.760 / 0.786 ms).  Mixed: 4 (128 registers); estimate, fit and backward pass of 300 k tracks
 // take 0.424 ms at 4, 0.449 ms at 5 (3.36 ms with the update in double).
+// All-double: blocks of one warp.  A few blocks of four per SM leave some SMs a whole block more to
+// do than others: 40 k tracks (1252 warps) estimated, fitted and carried back in 1.38 ms with 128
+// threads, 1.21 ms with 64, 1.17 ms with 32; 200 k tracks take 4.99 ms with any.
 constexpr int kFitThreads = 128;
+constexpr int kFitThreadsF64 = 32;
 template <class R, class U> struct FitMinBlocks {
     static constexpr int value = sizeof(R) == 8 ? 1 : sizeof(U) == 4 ? 7 : 4;
 };
@@ -795,10 +815,12 @@ __device__ __forceinline__ void fit_layers(const FitGeom &g, const tkf_hits &h, 
     int hid = first <= last ? hit_at(first) : -1;
     int hid1 = first + 1 <= last ? hit_at(first + 1) : -1;
     HitRec<R> cur = load_hit<R>(h, hid);
+    Trig<R> trig;
+    if (sizeof(R) == 8 && prop_first) trig = trig_of(p);
     for (int l = first; l <= last && status == 0; ++l) {
         const HitRec<R> nxt = load_hit<R>(h, hid1);
         const int hid2 = l + 2 <= last ? hit_at(l + 2) : -1;
-        if ((l > first || prop_first) && !to_layer<R, kDisk>(g, l, p, P, target_radius<R>(g, h, l, hid, cur), kb)) {
+        if ((l > first || prop_first) && !to_layer<R, kDisk>(g, l, p, P, target_radius<R>(g, h, l, hid, cur), kb, trig)) {
             status = TKF_TRACK_NOREACH;
             break;
         }
@@ -816,8 +838,7 @@ __device__ __forceinline__ void fit_layers(const FitGeom &g, const tkf_hits &h, 
             chi2 += dc2;
             nh += 1;
         }
-        if (l < g.L - 1)
-            scatter<R>(p, P, gpick<R>(g.xx0_f[l], g.xx0[l]), mass, kDisk && ((g.disk_mask >> l) & 1u));
+        if (l < g.L - 1) scatter_at<R>(g, l, p, P, mass, kDisk && ((g.disk_mask >> l) & 1u), trig);
         cur = nxt;
         hid = hid1;
         hid1 = hid2;
@@ -937,10 +958,11 @@ __global__ void __launch_bounds__(kFitThreads, (FitMinBlocks<R, U>::value)) k_fi
     int hid = last >= first ? hit_idx[last * si + i] : -1;
     int hid1 = last - 1 >= first ? hit_idx[(last - 1) * si + i] : -1;
     HitRec<R> cur = load_hit<R>(h, hid);
+    Trig<R> trig;  // formed by the first layer's scattering
     for (int l = last; l >= first && status == 0; --l) {
         const HitRec<R> nxt = load_hit<R>(h, hid1);
         const int hid2 = l - 2 >= first ? hit_idx[(l - 2) * si + i] : -1;
-        if (l < last && !to_layer<R, kDisk, kPropIn>(g, l, p, P, target_radius<R>(g, h, l, hid, cur), kb)) {
+        if (l < last && !to_layer<R, kDisk, kPropIn>(g, l, p, P, target_radius<R>(g, h, l, hid, cur), kb, trig)) {
             status = TKF_TRACK_NOREACH;
             break;
         }
@@ -958,7 +980,7 @@ __global__ void __launch_bounds__(kFitThreads, (FitMinBlocks<R, U>::value)) k_fi
             chi2 += dc2;
             nh += 1;
         }
-        scatter<R>(p, P, gpick<R>(g.xx0_f[l], g.xx0[l]), mass, kDisk && ((g.disk_mask >> l) & 1u));
+        scatter_at<R>(g, l, p, P, mass, kDisk && ((g.disk_mask >> l) & 1u), trig);
         cur = nxt;
         hid = hid1;
         hid1 = hid2;
@@ -1398,11 +1420,11 @@ int tkf::fit_tracks(tkf_ctx *ctx, const tkf_hits *hits, const tkf_tracks *init, 
     if (init->n == 0) return TKF_OK;
     const int32_t *hidx = hit_idx ? hit_idx : init->hit_idx;
     const FitGeom g = fit_geom(ctx);
-    const int nb = (init->n + 127) / 128;
+    const int nn = init->n, th = ctx->cfg.precision == TKF_FP64 ? kFitThreadsF64 : kFitThreads;
     cudaStream_t s = (cudaStream_t)stream;
     const int pf = continue_fit ? 1 : 0;
     auto go = [&](auto kern) {
-        kern<<<nb, kFitThreads, 0, s>>>(g, *hits, *init, hidx, first_layer, last_layer, pf, *out, ctx->d_err);
+        kern<<<(nn + th - 1) / th, th, 0, s>>>(g, *hits, *init, hidx, first_layer, last_layer, pf, *out, ctx->d_err);
     };
     const bool dk = g.disk_mask != 0;
     switch (ctx->cfg.precision) {
@@ -1429,10 +1451,10 @@ int tkf::fit_backward(tkf_ctx *ctx, const tkf_hits *hits, const tkf_tracks *init
     if (init->n == 0) return TKF_OK;
     const int32_t *hidx = hit_idx ? hit_idx : init->hit_idx;
     const FitGeom g = fit_geom(ctx);
-    const int nb = (init->n + 127) / 128;
+    const int nn = init->n, th = ctx->cfg.precision == TKF_FP64 ? kFitThreadsF64 : kFitThreads;
     cudaStream_t s = (cudaStream_t)stream;
     auto go = [&](auto kern, auto scale) {
-        kern<<<nb, kFitThreads, 0, s>>>(g, *hits, *init, hidx, last_layer, first_layer, scale, *out, ctx->d_err);
+        kern<<<(nn + th - 1) / th, th, 0, s>>>(g, *hits, *init, hidx, last_layer, first_layer, scale, *out, ctx->d_err);
     };
     const bool dk = g.disk_mask != 0;
     const float sf = (float)cov_scale;
@@ -1460,9 +1482,9 @@ int tkf::seed_and_fit(tkf_ctx *ctx, const tkf_hits *hits, const int32_t *seed_hi
         return set_err(ctx, TKF_ERR_INVALID, "need 0 <= last_layer < n_layers");
     if (out->n == 0) return TKF_OK;
     const FitGeom g = fit_geom(ctx);
-    const int nb = (out->n + 127) / 128;
+    const int nn = out->n, th = ctx->cfg.precision == TKF_FP64 ? kFitThreadsF64 : kFitThreads;
     cudaStream_t s = (cudaStream_t)stream;
-    auto go = [&](auto kern) { kern<<<nb, kFitThreads, 0, s>>>(g, *hits, seed_hits, last_layer, *out, ctx->d_err); };
+    auto go = [&](auto kern) { kern<<<(nn + th - 1) / th, th, 0, s>>>(g, *hits, seed_hits, last_layer, *out, ctx->d_err); };
     const bool dk = g.disk_mask != 0;
     switch (ctx->cfg.precision) {
     case TKF_FP32: dk ? go(k_seed_fit<float, float, true>) : go(k_seed_fit<float, float, false>); break;
