@@ -90,22 +90,45 @@ __device__ __forceinline__ float eta_of(float z, float r)
     return copysignf(fast_log(at + sqrtf(at * at + 1.f)), t);
 }
 
-__device__ __forceinline__ int hit_bin(const IndexGeom &g, int l, float x, float y, float z)
+// eta bin of a hit: on a cylinder eta of the layer's radius; on an endcap disk of the hit's own radius
+__device__ __forceinline__ int hit_eta_bin(const IndexGeom &g, float radius, bool disk, float x, float y, float z)
 {
-    // on a cylinder eta of the layer's radius; on an endcap disk of the hit's own radius
-    const float r = (g.disk_mask >> l) & 1u ? sqrtf(x * x + y * y) : g.radius[l];
-    int eb = (int)floorf((eta_of(z, r) - g.eta_min) * g.inv_eta_w);
-    eb = eb < 0 ? 0 : (eb >= g.n_eta ? g.n_eta - 1 : eb);
-    int pb = (int)floorf(phi_coord(g, x, y));
-    pb = pb < 0 ? 0 : (pb >= g.n_phi ? g.n_phi - 1 : pb);
-    return eb * g.n_phi + pb;
+    const float r = disk ? sqrtf(x * x + y * y) : radius;
+    const int eb = (int)floorf((eta_of(z, r) - g.eta_min) * g.inv_eta_w);
+    return eb < 0 ? 0 : (eb >= g.n_eta ? g.n_eta - 1 : eb);
 }
 
-// phi sub-bin (0..kSubBins-1) of a hit inside its phi bin pb, from the same phi coordinate
+__device__ __forceinline__ int clamp_phi_bin(const IndexGeom &g, float coord)
+{
+    const int pb = (int)floorf(coord);
+    return pb < 0 ? 0 : (pb >= g.n_phi ? g.n_phi - 1 : pb);
+}
+
+__device__ __forceinline__ int hit_bin(const IndexGeom &g, int l, float x, float y, float z)
+{
+    return hit_eta_bin(g, g.radius[l], (g.disk_mask >> l) & 1u, x, y, z) * g.n_phi +
+           clamp_phi_bin(g, phi_coord(g, x, y));
+}
+
+// phi sub-bin (0..kSubBins-1) of a hit at azimuth phi = a - pi inside its phi bin pb; the fraction of
+// the bin is one fused operation, so that every kernel puts a hit at a sixteenth's edge on the same side
+__device__ __forceinline__ int sub_of(const IndexGeom &g, float a, int pb)
+{
+    const int s = (int)floorf(fmaf(a, g.phi_scale, -(float)pb) * (float)kSubBins);
+    return s < 0 ? 0 : (s >= kSubBins ? kSubBins - 1 : s);
+}
+
 __device__ __forceinline__ int hit_sub(const IndexGeom &g, float x, float y, int pb)
 {
-    const int s = (int)floorf((phi_coord(g, x, y) - (float)pb) * (float)kSubBins);
-    return s < 0 ? 0 : (s >= kSubBins ? kSubBins - 1 : s);
+    return sub_of(g, atan2f(y, x) + (float)kPi, pb);
+}
+
+// bin and phi sixteenth of a hit, bin * kSubBins + sixteenth
+__device__ __forceinline__ unsigned hit_key(const IndexGeom &g, float radius, bool disk, float x, float y, float z)
+{
+    const float a = atan2f(y, x) + (float)kPi;
+    const int pb = clamp_phi_bin(g, a * g.phi_scale);
+    return (unsigned)((hit_eta_bin(g, radius, disk, x, y, z) * g.n_phi + pb) * kSubBins + sub_of(g, a, pb));
 }
 
 // key = ((event * L + layer) * n_bins + bin); counts per key.  The largest variances of each
@@ -395,10 +418,10 @@ __device__ __forceinline__ void sort_bins_warp(const IndexGeom &g, int b, int b_
     }
 }
 
-// Bin order of the whole index in one launch (used when an event's bins do not fit the
-// shared memory of the per-event kernel below): each warp takes kSortBinsPerWarp bins.  Held to
-// 5 blocks per SM (51 registers): 1.90 ms for the 640-event index against 2.08 ms at its natural
-// 64 registers and 4 blocks (6 blocks: 1.97 ms, with more spills), the same index.
+// Bin order of the whole index in one launch (the multi-launch path): each warp takes
+// kSortBinsPerWarp bins.  Held to 5 blocks per SM (51 registers): 1.90 ms for the 640-event index
+// against 2.08 ms at its natural 64 registers and 4 blocks (6 blocks: 1.97 ms, with more spills), the
+// same index.
 #ifndef TKF_SORT_MINBLOCKS
 #define TKF_SORT_MINBLOCKS 5
 #endif
@@ -419,190 +442,349 @@ k_bin_sort(const IndexGeom g, const int *bin_off, const int *ev_off, int n_bins_
         [](int k) { return k; }, s_key[w], s_bin[w], s_off[w], hxyzi, hvar, bin_sub, pos_of_hit);
 }
 
-// Order in which the per-event blocks below take the events: largest first (so that the
-// big events of a lognormal mix start early instead of trailing the launch); the rank of
-// event e counts the events larger than it, or as large with a smaller index.  Up to
-// kOrderMax events (beyond that the input order is kept).
-constexpr int kOrderMax = 4096;
+// ------------------------------------------------------------------ hit index, one block per layer of an event
+//
+// The segment of an (event, layer) holds a few thousand hits, and its place in the index is known
+// once the event's hits per layer are.  So k_index_layers counts those (reading the layers alone,
+// 4 bytes a hit), and one block of k_index_segment then does everything for its segment: counts per
+// phi sixteenth of every bin in shared memory, their scan (from which the bin tables follow), and
+// every hit straight to its place.  Positions are read twice (the second time from L2), variances
+// once, everything else is written once: 52 bytes a hit from and to HBM where counting, placing and
+// ordering in separate kernels moved 124.
 
-__global__ void __launch_bounds__(1024) k_event_order(const int *ev_off, int n_events, int *perm)
+// Hits of each (event, layer): count, runs of consecutive hits on the layer, and the first hit of
+// (any) one of them; one block per event.  Copies the event offsets into the index.
+constexpr int kLayerThreads = 1024;
+__global__ void __launch_bounds__(kLayerThreads) k_index_layers(const IndexGeom g, const tkf_hits h, int *ev_off,
+                                                                int *seg_count, int *seg_runs, int *seg_start, int *err)
 {
-    __shared__ int s_size[kOrderMax];
-    if (n_events > kOrderMax) {
-        for (int e = threadIdx.x; e < n_events; e += blockDim.x) perm[e] = e;
-        return;
-    }
-    for (int e = threadIdx.x; e < n_events; e += blockDim.x) s_size[e] = ev_off[e + 1] - ev_off[e];
-    __syncthreads();
-    for (int e = threadIdx.x; e < n_events; e += blockDim.x) {
-        const int se = s_size[e];
-        int rank = 0;
-        for (int f = 0; f < n_events; ++f) {
-            const int sf = s_size[f];
-            rank += sf > se || (sf == se && f < e);
-        }
-        perm[rank] = e;
-    }
-}
-
-// Folds a thread's running variance maxima of layer l (float bits of non-negative values, so
-// integer order is value order) into the block's maxima; l < 0: nothing held.
-__device__ __forceinline__ void var_flush(int *s_var, int l, int mu, int mv)
-{
-    if (l < 0) return;
-    atomicMax(&s_var[2 * l], mu);
-    atomicMax(&s_var[2 * l + 1], mv);
-}
-
-// The bins of one event in one block (one block per event, events taken in the order perm),
-// with the event's bin counters in shared memory: (1) count the hits per (layer, eta bin, phi
-// bin) and reduce the largest variances per layer; (2) exclusive scan of the counts ->
-// bin_off (the event's hits keep their place [event_off[e], event_off[e+1]) in the index);
-// (3) place every hit into its bin (a shared-memory cursor per bin).  k_bin_sort then orders
-// the bins.  The same bins and offsets as the multi-launch path.
-// The per-event kernels take a batch of at least TKF_INDEX_EVENTS_PER_SM events per SM; smaller
-// batches are spread over every SM by the multi-launch kernels.  Measured on the batched workload
-// (same indices): multi-launch 0.75 / 0.86 ms at 160 / 200 events against 0.91 / 0.98 ms per event,
-// per event 1.18 / 1.45 / 1.90 ms at 320 / 480 / 640 events against 1.23 / 1.85 / 2.62 ms.
-#ifndef TKF_INDEX_EVENTS_PER_SM
-#define TKF_INDEX_EVENTS_PER_SM 2
-#endif
-constexpr int kEventThreads = 1024;  // 512-thread blocks, two per SM: 2.46 ms against 1.88 ms (640 events)
-constexpr int kEventWarps = kEventThreads / 32;
-constexpr int kEventUnroll = 4;
-
-__global__ void __launch_bounds__(kEventThreads)
-k_index_event(const IndexGeom g, const tkf_hits h, const int *perm, int n_bins_total, float4 *hxyzi, float2 *hvar,
-              int *bin_off, float2 *var_max, int *err)
-{
-    extern __shared__ int s_cnt[];  // [L * n_bins]: counts, then bin offsets / cursors
-    __shared__ int s_var[2 * TKF_MAX_LAYERS];
-    __shared__ int s_part[kEventWarps];
-    const unsigned full = 0xffffffffu;
-    const int e = perm[blockIdx.x], tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    int cur_l = -1, mu = 0, mv = 0;  // this thread's layer and its largest variances (float bits)
-    const int nb_ev = g.L * g.n_bins;
+    __shared__ int s_cnt[TKF_MAX_LAYERS], s_runs[TKF_MAX_LAYERS], s_start[TKF_MAX_LAYERS];
+    const int e = blockIdx.x, tid = threadIdx.x;
     const int h0 = h.event_off[e], h1 = h.event_off[e + 1];
-    if (tid == 0 && h1 - h0 > kMaxHitsPerEvent) atomicOr(err, kErrTooManyHits);  // 23-bit local ids
-    for (int k = tid; k < nb_ev; k += kEventThreads) s_cnt[k] = 0;
-    if (tid < 2 * g.L) s_var[tid] = 0;
+    if (tid < g.L) s_cnt[tid] = s_runs[tid] = s_start[tid] = 0;
+    if (tid == 0) {
+        ev_off[e] = h0;
+        if (e == g.n_events - 1) ev_off[e + 1] = h1;
+        if (h1 - h0 > kMaxHitsPerEvent) atomicOr(err, kErrTooManyHits);  // 23-bit local ids
+    }
     __syncthreads();
-    // (1) counts and variance maxima; kEventUnroll hits per thread and pass, loaded together
-    for (int i0 = h0; i0 < h1; i0 += kEventThreads * kEventUnroll) {
-        int l[kEventUnroll];
-        float x[kEventUnroll], y[kEventUnroll], z[kEventUnroll], vu[kEventUnroll], vv[kEventUnroll];
+    // four consecutive hits per thread, read as one word where the array is aligned to it; four such
+    // words in flight (the largest event's block is the kernel's tail)
+    const bool aligned = ((size_t)h.layer & 15) == 0;
+    constexpr int U = 4;
+    for (int p0 = (h0 & ~3) + 4 * tid; p0 < h1; p0 += U * 4 * kLayerThreads) {
+        int l[U][6];  // layers of hits i0 - 1 .. i0 + 4
 #pragma unroll
-        for (int u = 0; u < kEventUnroll; ++u) {
-            const int i = i0 + tid + u * kEventThreads;
-            const int j = i < h1 ? i : h0;  // a valid index (the event is not empty here)
-            l[u] = h.layer[j];
-            x[u] = h.x[j];
-            y[u] = h.y[j];
-            z[u] = h.z[j];
-            vu[u] = h.var_u[j];
-            vv[u] = h.var_v[j];
+        for (int v = 0; v < U; ++v) {
+            const int i0 = p0 + v * 4 * kLayerThreads;
+            if (aligned && i0 + 4 <= h.n) {
+                const int4 q = __ldg((const int4 *)(h.layer + i0));
+                l[v][1] = q.x;
+                l[v][2] = q.y;
+                l[v][3] = q.z;
+                l[v][4] = q.w;
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) l[v][u + 1] = i0 + u < h1 ? __ldg(&h.layer[i0 + u]) : -1;
+            }
+            l[v][0] = i0 > h0 && i0 <= h1 ? __ldg(&h.layer[i0 - 1]) : -1;
+            l[v][5] = i0 + 4 < h1 ? __ldg(&h.layer[i0 + 4]) : -1;
         }
 #pragma unroll
-        for (int u = 0; u < kEventUnroll; ++u) {
-            const bool in = i0 + tid + u * kEventThreads < h1;
-            const bool ok = in && l[u] >= 0 && l[u] < g.L;
-            if (ok) {
-                atomicAdd(&s_cnt[l[u] * g.n_bins + hit_bin(g, l[u], x[u], y[u], z[u])], 1);
-                if (l[u] != cur_l) {  // hits usually come grouped by layer: rare
-                    var_flush(s_var, cur_l, mu, mv);
-                    cur_l = l[u];
-                    mu = mv = 0;
+        for (int v = 0; v < U; ++v) {
+            const int i0 = p0 + v * 4 * kLayerThreads;
+            // most words lie inside a run: nothing to record
+            if (i0 > h0 && i0 + 4 < h1 && l[v][0] == l[v][1] && l[v][1] == l[v][2] && l[v][2] == l[v][3] &&
+                l[v][3] == l[v][4] && l[v][4] == l[v][5] && l[v][1] >= 0 && l[v][1] < g.L)
+                continue;
+#pragma unroll
+            for (int u = 1; u < 5; ++u) {
+                const int i = i0 + u - 1, c = l[v][u];
+                if (i < h0 || i >= h1) continue;
+                if (c < 0 || c >= g.L) {
+                    atomicOr(err, kErrBadLayer);
+                    continue;
                 }
-                mu = max(mu, __float_as_int(fmaxf(vu[u], 0.f)));
-                mv = max(mv, __float_as_int(fmaxf(vv[u], 0.f)));
-            } else if (in) {
-                atomicOr(err, kErrBadLayer);
+                if (c != l[v][u - 1] || i == h0) {  // a run's length is its end minus its start
+                    atomicAdd(&s_runs[c], 1);
+                    atomicAdd(&s_cnt[c], -i);
+                    s_start[c] = i;
+                }
+                if (c != l[v][u + 1] || i == h1 - 1) atomicAdd(&s_cnt[c], i + 1);
             }
         }
     }
-    {  // the last running maxima, one atomic per layer and warp
-        const unsigned grp = __match_any_sync(full, cur_l);
-        const int ru = __reduce_max_sync(grp, (unsigned)mu), rv = __reduce_max_sync(grp, (unsigned)mv);
-        if (lane == __ffs(grp) - 1) var_flush(s_var, cur_l, ru, rv);
-    }
     __syncthreads();
-    // (2) exclusive scan: thread t owns the contiguous chunk [t * per, (t + 1) * per)
-    const int per = (nb_ev + kEventThreads - 1) / kEventThreads;
-    const int c0 = min(tid * per, nb_ev), c1 = min(c0 + per, nb_ev);
-    int sum = 0;
-    for (int k = c0; k < c1; ++k) sum += s_cnt[k];
-    int incl = sum;
+    if (tid < g.L) {
+        seg_count[e * g.L + tid] = s_cnt[tid];
+        seg_runs[e * g.L + tid] = s_runs[tid];
+        seg_start[e * g.L + tid] = s_start[tid];
+    }
+}
+
+constexpr int kSegMaxBins = 4096;  // a bin's sixteenth in 16 bits
+constexpr int kSegThreads = 768, kSegThreadsBig = 1024;
+constexpr size_t kSegSmem = 112 * 1024, kSegSmemBig = 226 * 1024;  // two blocks per SM, one
+
+// Shared memory of a segment: a 16-bit counter for each sixteenth of each bin and one more (padded to
+// whole 16-byte words), and 4 bytes for each hit.
+__host__ __device__ __forceinline__ int seg_words(int n_bins) { return (n_bins * kSubBins + 8) / 8; }
+int segment_cap(int n_bins, size_t smem) { return ((int)smem - 16 * seg_words(n_bins)) / 4; }
+
+__device__ __forceinline__ unsigned half16(const unsigned *w, unsigned k) { return (w[k >> 1] >> (16 * (k & 1))) & 0xFFFFu; }
+
+// One pass of a segment's hits through its block: f(position in the segment, x, y, z), U hits per thread
+// loaded together.
+template <int T, class F> __device__ __forceinline__ void for_hits(const tkf_hits &h, int i0, int cnt, F f)
+{
+    constexpr int U = 4;
+    for (int j0 = threadIdx.x; j0 < cnt; j0 += U * T) {
+        float x[U], y[U], z[U];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(full, incl, o);
-        if (lane >= o) incl += t;
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + min(j0 + u * T, cnt - 1);
+            x[u] = h.x[i];
+            y[u] = h.y[i];
+            z[u] = h.z[i];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j0 + u * T < cnt) f(j0 + u * T, x[u], y[u], z[u]);
     }
-    if (lane == 31) s_part[w] = incl;
-    __syncthreads();
-    if (w == 0) {
-        int x = lane < kEventWarps ? s_part[lane] : 0;
+}
+
+// The segment of one (event, layer).  A launch takes the segments of one run with lo < hits <= cap,
+// held in shared memory; the last launch (kLast) also those that are larger or whose hits are not
+// consecutive: only their bins are counted there, the hits' keys live in pos_of_hit and their order
+// words in hvar until the final positions are known, and hits on other layers in between are passed
+// over.
+//
+// What bounds it: the latency of its phases (loads, counting, scan, tables, placing, each behind a
+// barrier) with 73 % of the warps resident and 40 % issue; 512 events (23.5 M hits) move 1.7 GB in 0.70
+// ms, with k_index_layers (36 us, the largest event's block) included.  Before, in 1.45 ms: one block
+// per event counting and placing (0.92 ms), then an ordering pass over the whole index (0.48 ms).
+// Measured and not taken: hits ordered in their bins by order words (rank loops over the bin) 0.87
+// ms; the same with a segment's bins shared out over blocks of 5000 hits 1.24 ms (every block bins
+// every hit); tables written by the scan's threads 0.88 ms (uncoalesced); 512 / 1024 threads 0.75 /
+// 0.73 ms.
+template <int T, int kPerSM, bool kLast>
+__global__ void __launch_bounds__(T, kPerSM)
+k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int *__restrict__ seg_count,
+                const int *__restrict__ seg_runs, const int *__restrict__ seg_start, int lo, int cap, float4 *hxyzi,
+                float2 *hvar, uint4 *bin_sub, int *pos_of_hit, int *bin_off, float2 *var_max)
+{
+    extern __shared__ uint4 s_words[];
+    __shared__ int s_part[T / 32], s_mu, s_mv;
+    const unsigned full = 0xffffffffu;
+    const int seg = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int cnt = seg_count[seg];
+    const bool grouped = seg_runs[seg] <= 1, fast = grouped && cnt <= cap && cnt < 65536;
+    if (fast ? cnt <= lo : !kLast) return;
+    const int e = seg / g.L, l = seg - e * g.L;
+    const int h0 = h.event_off[e];
+    int base = h0;
+    for (int k = 0; k < l; ++k) base += seg_count[e * g.L + k];
+    const int i0 = grouped ? seg_start[seg] : h0, i1 = grouped ? i0 + cnt : h.event_off[e + 1];
+    const float rl = g.radius[l];
+    const bool disk = (g.disk_mask >> l) & 1u;
+    const size_t b0 = (size_t)seg * g.n_bins;
+    if (tid == 0) s_mu = s_mv = 0;
+    if (seg == g.n_events * g.L - 1 && tid == 0) bin_off[b0 + g.n_bins] = base + cnt;
+    float mu = 0.f, mv = 0.f;
+    if (fast) {
+        const int nw = seg_words(g.n_bins);
+        unsigned *s_cell = (unsigned *)s_words;  // two cells a word
+        unsigned short *s_key = (unsigned short *)(s_words + nw), *s_ord = s_key + cap;
+        for (int k = tid; k < nw; k += T) s_words[k] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        // (1) the sixteenth of every hit; hits per sixteenth
+        for_hits<T>(h, i0, cnt, [&](int j, float x, float y, float z) {
+            const unsigned key = hit_key(g, rl, disk, x, y, z);
+            s_key[j] = (unsigned short)key;
+            atomicAdd(&s_cell[key >> 1], key & 1 ? 0x10000u : 1u);
+        });
+        __syncthreads();
+        // (2) inclusive scan: the end of every sixteenth; thread t owns a contiguous chunk of words, an
+        // odd number of them (a multiple of 8 would put every lane's words in the same banks)
+        const int per = ((nw + T - 1) / T) | 1, c0 = min(tid * per, nw), c1 = min(c0 + per, nw);
+        unsigned sum = 0;  // both halves at once: no carry, the segment has fewer than 2^16 hits
+        for (int k = c0; k < c1; ++k) {
+            const uint4 q = s_words[k];
+            sum += q.x + q.y + q.z + q.w;
+        }
+        const int mine = (int)((sum & 0xFFFFu) + (sum >> 16));
+        int incl = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(full, x, o);
-            if (lane >= o) x += t;
+            const int t = __shfl_up_sync(full, incl, o);
+            if (lane >= o) incl += t;
         }
-        if (lane < kEventWarps) s_part[lane] = x;  // inclusive warp totals
+        if (lane == 31) s_part[w] = incl;
+        __syncthreads();
+        unsigned run = (unsigned)(incl - mine);
+        for (int k = 0; k < w; ++k) run += (unsigned)s_part[k];
+        auto ends = [&](unsigned c) {  // both cells' ends from their counts
+            const unsigned a = run + (c & 0xFFFFu);
+            run = a + (c >> 16);
+            return a | (run << 16);
+        };
+        for (int k = c0; k < c1; ++k) {
+            uint4 q = s_words[k];
+            q.x = ends(q.x);
+            q.y = ends(q.y);
+            q.z = ends(q.z);
+            q.w = ends(q.w);
+            s_words[k] = q;
+        }
+        __syncthreads();
+        // (3) hits into their sixteenths, from the end down: the cells then hold the starts
+        for (int j = tid; j < cnt; j += T) {
+            const unsigned key = s_key[j], sh = 16 * (key & 1);
+            const unsigned old = atomicSub(&s_cell[key >> 1], 1u << sh);
+            s_ord[((old >> sh) & 0xFFFFu) - 1] = (unsigned short)j;
+        }
+        __syncthreads();
+        // (4) the bin tables: a bin's sixteenths are 8 words; their starts relative to the bin's, as bytes
+        for (int b = tid; b < g.n_bins; b += T) {
+            const uint4 q0 = s_words[2 * b], q1 = s_words[2 * b + 1];
+            const unsigned a = q0.x & 0xFFFFu, n = half16(s_cell, (b + 1) * kSubBins) - a;
+            bin_off[b0 + b] = base + (int)a;
+            const unsigned aa = a | (a << 16);  // no borrow: starts do not decrease
+            auto bytes = [](unsigned u, unsigned v, unsigned x) {  // halves u.hi, v.lo, v.hi, x.lo
+                return __byte_perm(__byte_perm(u, v, 0x0642), x, 0x4210);
+            };
+            const unsigned d0 = q0.x - aa, d1 = q0.y - aa, d2 = q0.z - aa, d3 = q0.w - aa;
+            const unsigned d4 = q1.x - aa, d5 = q1.y - aa, d6 = q1.z - aa, d7 = q1.w - aa;
+            uint4 sub = make_uint4(bytes(d0, d1, d2), bytes(d2, d3, d4), bytes(d4, d5, d6), bytes(d6, d7, 0u));
+            if (n > 255u) sub = make_uint4(~0u, ~0u, ~0u, ~0u);
+            bin_sub[b0 + b] = sub;
+        }
+        // (5) the hits to their places: a sixteenth's hits in the order of their ids
+        auto place = [&](int j, float x, float y, float z) {
+            const unsigned key = s_key[j];
+            const int a0 = (int)half16(s_cell, key), a1 = (int)half16(s_cell, key + 1);
+            int pos = base + a0;
+            if (a1 - a0 > 1)
+                for (int t = a0; t < a1; ++t) pos += s_ord[t] < j;
+            const int i = i0 + j;
+            const float vu = h.var_u[i], vv = h.var_v[i];
+            hxyzi[pos] = make_float4(x, y, z, __int_as_float(i - h0));
+            hvar[pos] = make_float2(vu, vv);
+            pos_of_hit[i] = pos;
+            mu = fmaxf(mu, vu);
+            mv = fmaxf(mv, vv);
+        };
+        for_hits<T>(h, i0, cnt, place);
+    } else {
+        int *s_bin = (int *)s_words;  // counts, then cursors: start of a bin, then its end
+        unsigned *g_ord = (unsigned *)(hvar + base);  // order word (sixteenth, id) q at 2 q
+        for (int b = tid; b < g.n_bins; b += T) s_bin[b] = 0;
+        __syncthreads();
+        for (int i = i0 + tid; i < i1; i += T) {
+            if (h.layer[i] != l) continue;
+            const unsigned key = hit_key(g, rl, disk, h.x[i], h.y[i], h.z[i]);
+            pos_of_hit[i] = (int)key;
+            atomicAdd(&s_bin[key / kSubBins], 1);
+        }
+        __syncthreads();
+        const int per = (g.n_bins + T - 1) / T, c0 = min(tid * per, g.n_bins), c1 = min(c0 + per, g.n_bins);
+        int sum = 0;
+        for (int b = c0; b < c1; ++b) sum += s_bin[b];
+        int incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(full, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) s_part[w] = incl;
+        __syncthreads();
+        int run = incl - sum;
+        for (int k = 0; k < w; ++k) run += s_part[k];
+        for (int b = c0; b < c1; ++b) {
+            const int c = s_bin[b];
+            s_bin[b] = run;
+            run += c;
+        }
+        __syncthreads();
+        for (int i = i0 + tid; i < i1; i += T) {
+            if (h.layer[i] != l) continue;
+            const unsigned key = (unsigned)pos_of_hit[i];
+            g_ord[2 * (size_t)atomicAdd(&s_bin[key / kSubBins], 1)] =
+                ((key & (kSubBins - 1)) << 23) | ((unsigned)(i - h0) & 0x7FFFFFu);
+        }
+        __syncthreads();
+        for (int b = tid; b < g.n_bins; b += T) {
+            const int a0 = b ? s_bin[b - 1] : 0, a1 = s_bin[b];
+            bin_off[b0 + b] = base + a0;
+            bin_sub[b0 + b] = sub_starts([&](int t) { return (int)g_ord[2 * (size_t)t]; }, a0, a1);
+        }
+        for (int i = i0 + tid; i < i1; i += T) {
+            if (h.layer[i] != l) continue;
+            const unsigned key = (unsigned)pos_of_hit[i], b = key / kSubBins;
+            const unsigned word = ((key & (kSubBins - 1)) << 23) | ((unsigned)(i - h0) & 0x7FFFFFu);
+            const int a0 = b ? s_bin[b - 1] : 0, a1 = s_bin[b];
+            int pos = base + a0;
+            for (int t = a0; t < a1; ++t) pos += g_ord[2 * (size_t)t] < word;
+            pos_of_hit[i] = pos;
+        }
+        __syncthreads();  // every word has been compared: hvar takes the variances
+        for (int i = i0 + tid; i < i1; i += T) {
+            if (h.layer[i] != l) continue;
+            const int pos = pos_of_hit[i];
+            const float vu = h.var_u[i], vv = h.var_v[i];
+            hxyzi[pos] = make_float4(h.x[i], h.y[i], h.z[i], __int_as_float(i - h0));
+            hvar[pos] = make_float2(vu, vv);
+            mu = fmaxf(mu, vu);
+            mv = fmaxf(mv, vv);
+        }
+    }
+    // the largest variances (the order of non-negative floats is that of their bits)
+    const unsigned ru = __reduce_max_sync(full, __float_as_uint(mu)), rv = __reduce_max_sync(full, __float_as_uint(mv));
+    if (lane == 0) {
+        atomicMax(&s_mu, (int)ru);
+        atomicMax(&s_mv, (int)rv);
     }
     __syncthreads();
-    int run = incl - sum + (w > 0 ? s_part[w - 1] : 0);
-    const size_t gb0 = (size_t)e * nb_ev;
-    for (int k = c0; k < c1; ++k) {
-        const int c = s_cnt[k];
-        s_cnt[k] = run;
-        bin_off[gb0 + k] = h0 + run;
-        run += c;
-    }
-    if (e == g.n_events - 1 && tid == kEventThreads - 1) bin_off[n_bins_total] = h0 + run;
-    if (tid < g.L)
-        var_max[(size_t)e * g.L + tid] = make_float2(__int_as_float(s_var[2 * tid]), __int_as_float(s_var[2 * tid + 1]));
-    __syncthreads();
-    // (3) place the hits, kEventUnroll per thread and pass
-    for (int i0 = h0; i0 < h1; i0 += kEventThreads * kEventUnroll) {
-        int l[kEventUnroll];
-        float x[kEventUnroll], y[kEventUnroll], z[kEventUnroll], vu[kEventUnroll], vv[kEventUnroll];
-#pragma unroll
-        for (int u = 0; u < kEventUnroll; ++u) {
-            const int i = i0 + tid + u * kEventThreads;
-            const int j = i < h1 ? i : h0;
-            l[u] = h.layer[j];
-            x[u] = h.x[j];
-            y[u] = h.y[j];
-            z[u] = h.z[j];
-            vu[u] = h.var_u[j];
-            vv[u] = h.var_v[j];
-        }
-#pragma unroll
-        for (int u = 0; u < kEventUnroll; ++u) {
-            const int i = i0 + tid + u * kEventThreads;
-            if (i >= h1 || l[u] < 0 || l[u] >= g.L) continue;
-            const int pos = h0 + atomicAdd(&s_cnt[l[u] * g.n_bins + hit_bin(g, l[u], x[u], y[u], z[u])], 1);
-            hxyzi[pos] = make_float4(x[u], y[u], z[u], __int_as_float(i - h0));
-            hvar[pos] = make_float2(vu[u], vv[u]);
-        }
-    }
+    if (tid == 0) var_max[seg] = make_float2(__int_as_float(s_mu), __int_as_float(s_mv));
 }
 
-// Dynamic shared memory of k_index_event (the event's bin counters) allowed next to its
-// static arrays within one block's 227 KB; an index whose event bins need more takes the
-// multi-launch path.
-constexpr size_t kEventStaticSmem = (size_t)kEventWarps * 4 + 2 * TKF_MAX_LAYERS * 4;
-constexpr size_t kEventMaxDynSmem = 227 * 1024 - kEventStaticSmem - 1024;
-
-size_t index_event_smem(int n_layers, int n_bins)
+// Whether a batch is indexed by k_index_segment: its sixteenths fit 16 bits and its segments, on
+// average, a block's shared memory; otherwise the multi-launch kernels spread it over the GPU.  A
+// single event of 162 k hits (ten blocks) takes 56 us here and 84 us there, one of 270 k hits 121 us
+// there; 20 events of 67 k hits 57 and 143 us, 64 / 160 events 176 / 316 and 332 / 705 us.
+bool segment_index(int n_hits, size_t n_segs, int n_bins)
 {
-    const size_t bytes = (size_t)n_layers * n_bins * sizeof(int);
-    return bytes <= kEventMaxDynSmem ? bytes : 0;
+    return n_bins <= kSegMaxBins && n_bins >= 4 && (size_t)n_hits <= n_segs * 16384;
 }
 
-// Allows k_index_event its dynamic shared memory on the current device.
-cudaError_t index_event_prepare()
+// seg: 3 n_segs words of scratch.
+cudaError_t launch_segment_index(const IndexGeom &g, const tkf_hits &h, int sm_count, int *seg, int *ev_off,
+                                 float4 *hxyzi, float2 *hvar, uint4 *bin_sub, int *pos_of_hit, int *bin_off,
+                                 float2 *var_max, int *err, cudaStream_t s)
 {
-    return cudaFuncSetAttribute(k_index_event, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEventMaxDynSmem);
+    const unsigned n_segs = (unsigned)(g.n_events * g.L);
+    int *cnt = seg, *runs = seg + n_segs, *start = runs + n_segs;
+    k_index_layers<<<(unsigned)g.n_events, kLayerThreads, 0, s>>>(g, h, ev_off, cnt, runs, start, err);
+    int lo = -1;
+    auto take = [&](auto kern, int threads, size_t smem) {
+        const int hi = segment_cap(g.n_bins, smem);
+        kern<<<n_segs, threads, smem, s>>>(g, h, cnt, runs, start, lo, hi, hxyzi, hvar, bin_sub, pos_of_hit, bin_off,
+                                           var_max);
+        lo = std::max(hi, -1);
+    };
+    if ((int)n_segs > sm_count) take(k_index_segment<kSegThreads, 2, false>, kSegThreads, kSegSmem);
+    take(k_index_segment<kSegThreadsBig, 1, true>, kSegThreadsBig, kSegSmemBig);
+    return cudaGetLastError();
+}
+
+// Allows the segment kernels their dynamic shared memory on the current device.
+cudaError_t segment_index_prepare()
+{
+    const cudaError_t e = cudaFuncSetAttribute(k_index_segment<kSegThreads, 2, false>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSmem);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(k_index_segment<kSegThreadsBig, 1, true>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSmemBig);
 }
 
 unsigned sort_blocks(size_t n_bins)
@@ -1202,7 +1384,7 @@ int tkf_create(const tkf_config *cfg, tkf_ctx **out)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device);
     if (e == cudaSuccess) e = cudaMalloc((void **)&ctx->d_tile, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc((void **)&ctx->d_err, sizeof(int));
-    if (e == cudaSuccess) e = index_event_prepare();
+    if (e == cudaSuccess) e = segment_index_prepare();
     if (e == cudaSuccess) e = cudaMemset(ctx->d_err, 0, sizeof(int));
     if (e != cudaSuccess) {
         if (ctx->d_tile) cudaFree(ctx->d_tile);
@@ -1281,24 +1463,15 @@ int tkf_build_hit_index(tkf_ctx *ctx, const tkf_hits *hits, tkf_hit_index **out,
         idx->n_bins = NB;
         cudaStream_t s = (cudaStream_t)stream;
         const IndexGeom g = index_geom(c, hits->n_events);
-        TKF_CUDA(ctx, cudaMemcpyAsync(idx->ev_off, hits->event_off, (hits->n_events + 1) * sizeof(int),
-                                      cudaMemcpyDeviceToDevice, s));
-        // one block per event when the batch has enough events to fill the GPU twice and their
-        // bins fit a block's shared memory (set up by tkf_create); otherwise counts in global
-        // memory and every block on the hits of a few events
-        const size_t ev_smem = hits->n_events >= TKF_INDEX_EVENTS_PER_SM * ctx->sm_count ? index_event_smem(L, NB) : 0;
-        if (ev_smem) {
-            int *perm = idx->seg_base;  // >= n_events entries
-            k_event_order<<<1, 1024, 0, s>>>(hits->event_off, hits->n_events, perm);
-            k_index_event<<<(unsigned)hits->n_events, kEventThreads, ev_smem, s>>>(
-                g, *hits, perm, (int)n_bins, idx->hxyzi, idx->hvar, idx->bin_off, idx->var_max, ctx->d_err);
-            k_bin_sort<<<sort_blocks(n_bins), 32 * kSortWarps, 0, s>>>(g, idx->bin_off, idx->ev_off, (int)n_bins,
-                                                                       idx->hxyzi, idx->hvar, idx->bin_sub,
-                                                                       idx->pos_of_hit);
-            TKF_CUDA(ctx, cudaGetLastError());
+        if (segment_index(hits->n, n_segs, NB)) {
+            TKF_CUDA(ctx, launch_segment_index(g, *hits, ctx->sm_count, idx->counts, idx->ev_off, idx->hxyzi, idx->hvar,
+                                               idx->bin_sub, idx->pos_of_hit, idx->bin_off, idx->var_max, ctx->d_err,
+                                               s));
             *out = idx;
             return TKF_OK;
         }
+        TKF_CUDA(ctx, cudaMemcpyAsync(idx->ev_off, hits->event_off, (hits->n_events + 1) * sizeof(int),
+                                      cudaMemcpyDeviceToDevice, s));
         TKF_CUDA(ctx, cudaMemsetAsync(idx->counts, 0, n_bins * sizeof(int), s));
         TKF_CUDA(ctx, cudaMemsetAsync(idx->var_max, 0, n_segs * sizeof(float2), s));
         if (hits->n > 0) {
@@ -1667,7 +1840,7 @@ int noalloc_scratch(int **out, int *sm_count)
     if (!g_noalloc_addr[dev]) {
         int *p = nullptr;
         if (cudaGetSymbolAddress((void **)&p, g_noalloc_scratch) != cudaSuccess || !p) return TKF_ERR_CUDA;
-        if (index_event_prepare() != cudaSuccess) return TKF_ERR_CUDA;
+        if (segment_index_prepare() != cudaSuccess) return TKF_ERR_CUDA;
         if (cudaDeviceGetAttribute(&g_noalloc_sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return TKF_ERR_CUDA;
         g_noalloc_addr[dev] = p;
@@ -1712,18 +1885,14 @@ extern "C" int tkf_build_hit_index_noalloc(const tkf_config *cfg, const tkf_hits
     cudaStream_t s = (cudaStream_t)stream;
     float4 *hxyzi = (float4 *)out->hit_xyzi;
     float2 *hvar = (float2 *)out->hit_var;
+    if (segment_index(hits->n, n_segs, NB))
+        return launch_segment_index(g, *hits, n_sm, counts, out->event_off, hxyzi, hvar, (uint4 *)out->bin_sub,
+                                    out->pos_of_hit, out->bin_off, (float2 *)out->var_max, err, s) == cudaSuccess
+                   ? TKF_OK
+                   : TKF_ERR_CUDA;
     if (cudaMemcpyAsync(out->event_off, hits->event_off, (hits->n_events + 1) * sizeof(int), cudaMemcpyDeviceToDevice,
                         s) != cudaSuccess)
         return TKF_ERR_CUDA;
-    if (const size_t ev_smem = hits->n_events >= TKF_INDEX_EVENTS_PER_SM * n_sm ? index_event_smem(L, NB) : 0) {
-        // one block per event
-        k_event_order<<<1, 1024, 0, s>>>(hits->event_off, hits->n_events, seg_base);
-        k_index_event<<<(unsigned)hits->n_events, kEventThreads, ev_smem, s>>>(
-            g, *hits, seg_base, (int)n_bins, hxyzi, hvar, out->bin_off, (float2 *)out->var_max, err);
-        k_bin_sort<<<sort_blocks(n_bins), 32 * kSortWarps, 0, s>>>(g, out->bin_off, out->event_off, (int)n_bins, hxyzi,
-                                                                   hvar, (uint4 *)out->bin_sub, out->pos_of_hit);
-        return cudaGetLastError() == cudaSuccess ? TKF_OK : TKF_ERR_CUDA;
-    }
     if (cudaMemsetAsync(counts, 0, n_bins * sizeof(int), s) != cudaSuccess ||
         cudaMemsetAsync(out->var_max, 0, n_segs * 2 * sizeof(float), s) != cudaSuccess)
         return TKF_ERR_CUDA;
