@@ -7,9 +7,9 @@
 //   2. it scans the hits of its eta-phi window (CSR bins of the hit index), scores each by
 //      chi2 and keeps its own best-N branch keys in a register list; a candidate with no
 //      compatible hit contributes one hole key;
-//   3. the segment merges its lanes' lists: N rounds of a segmented warp-shuffle minimum give
-//      the seed's N best branches in rank order (the paper's "branching to explore multiple
-//      candidate tracks per seed" and the per-seed repacking of Sec. 3.2.1);
+//   3. the segment merges its lanes' lists into the seed's N best branches in rank order (the paper's
+//      "branching to explore multiple candidate tracks per seed" and the per-seed repacking of
+//      Sec. 3.2.1): N rounds of a segmented warp-shuffle minimum, or counting ranks in shared memory;
 //   4. the lane of rank r fetches its parent's predicted state with shuffles, applies the
 //      Kalman update (U = float or double) for a hit branch and the layer's scattering noise.
 // With hits off the layers' cylinders (kTwo) step 1 reaches the layer's average radius, step 2
@@ -56,31 +56,152 @@ __device__ __forceinline__ unsigned make_key32(int nhits, float chi2, int parent
 
 __device__ __forceinline__ float key_chi2(unsigned key) { return __uint_as_float(((key >> 4) & 0x7FFFFFu) << 8); }
 
-// A lane's branch list: its NMAX smallest keys in ascending order (lk), with their hit ids (lh);
-// a key equal to one already listed goes after it.
-template <int NMAX>
-__device__ __forceinline__ void list_insert32(unsigned (&lk)[NMAX], int (&lh)[NMAX], unsigned k, int h)
-{
+// A lane's branch list in registers: its NMAX smallest keys in ascending order (lk), with their hit
+// ids (lh); a key equal to one already listed goes after it.
+template <int NMAX> struct SortedList {
+    unsigned lk[NMAX];
+    int lh[NMAX];
+    __device__ __forceinline__ explicit SortedList(unsigned * = nullptr)
+    {
 #pragma unroll
-    for (int i = 0; i < NMAX; ++i) {
-        const bool lt = k < lk[i];
-        const unsigned k2 = lt ? lk[i] : k;
-        const int h2 = lt ? lh[i] : h;
-        lk[i] = lt ? k : lk[i];
-        lh[i] = lt ? h : lh[i];
-        k = k2;
-        h = h2;
+        for (int i = 0; i < NMAX; ++i) {
+            lk[i] = kEmpty32;
+            lh[i] = 0;
+        }
     }
+    __device__ __forceinline__ void push(unsigned k, int h)
+    {
+#pragma unroll
+        for (int i = 0; i < NMAX; ++i) {
+            const bool lt = k < lk[i];
+            const unsigned k2 = lt ? lk[i] : k;
+            const int h2 = lt ? lh[i] : h;
+            lk[i] = lt ? k : lk[i];
+            lh[i] = lt ? h : lh[i];
+            k = k2;
+            h = h2;
+        }
+    }
+    __device__ __forceinline__ void pop()
+    {
+#pragma unroll
+        for (int i = 0; i + 1 < NMAX; ++i) {
+            lk[i] = lk[i + 1];
+            lh[i] = lh[i + 1];
+        }
+        lk[NMAX - 1] = kEmpty32;
+    }
+};
+
+// The N smallest branches of a segment (N lanes from lane gbase of the warp on, r this lane's place),
+// from its lanes' lists: lane r gets the branch of rank r (kEmpty32: there are fewer); returns their
+// number.  N rounds of a segmented minimum over the lists' heads.
+template <int NMAX>
+__device__ __forceinline__ int merge_lists(SortedList<NMAX> &list, int N, int r, bool lane_ok, int lane, int gbase,
+                                           unsigned &mine, int &mine_h)
+{
+    mine = kEmpty32;
+    mine_h = 0;
+    int ns = 0;
+    for (int k = 0; k < N; ++k) {
+        if (!__any_sync(kFull, list.lk[0] != kEmpty32)) break;  // no segment has branches left
+        unsigned m = list.lk[0];
+        for (int off = 1; off < N; off <<= 1) {
+            const unsigned o = __shfl_down_sync(kFull, m, off);
+            if (r + off < N && o < m) m = o;
+        }
+        m = __shfl_sync(kFull, m, gbase);
+        // the winner is the lane whose rank is the key's parent field
+        const int hsel = __shfl_sync(kFull, list.lh[0], lane_ok ? gbase + (int)(m & 0xFu) : lane);
+        if (m != kEmpty32) {
+            if (list.lk[0] == m) list.pop();
+            if (r == k) {
+                mine = m;
+                mine_h = hsel;
+            }
+            ns = k + 1;
+        }
+    }
+    return ns;
 }
 
-template <int NMAX> __device__ __forceinline__ void list_pop32(unsigned (&lk)[NMAX], int (&lh)[NMAX])
-{
-#pragma unroll
-    for (int i = 0; i + 1 < NMAX; ++i) {
-        lk[i] = lk[i + 1];
-        lh[i] = lh[i + 1];
+// A lane's branch list in shared memory, in the order of the pushes: its NMAX smallest keys (of equal
+// ones the earlier).  Word i of the thread's column of the block's planes (T words apart) is key i,
+// word NMAX + i its hit id.
+template <int NMAX, int T> struct ColumnList {
+    unsigned *col;
+    int n = 0;
+    __device__ __forceinline__ explicit ColumnList(unsigned *c) : col(c) {}
+    __device__ __forceinline__ void push(unsigned k, int h)
+    {
+        if (n == NMAX) {  // rare: the largest key (the last of equals) makes room
+            int m = 0;
+            unsigned km = col[0];
+            for (int i = 1; i < NMAX; ++i)
+                if (col[i * T] >= km) {
+                    km = col[i * T];
+                    m = i;
+                }
+            if (k >= km) return;
+            for (int i = m; i + 1 < NMAX; ++i) {
+                col[i * T] = col[(i + 1) * T];
+                col[(NMAX + i) * T] = col[(NMAX + i + 1) * T];
+            }
+            n = NMAX - 1;
+        }
+        col[n * T] = k;
+        col[(NMAX + n) * T] = (unsigned)h;
+        ++n;
     }
-    lk[NMAX - 1] = kEmpty32;
+};
+
+// The same from lists in shared memory (lists of more than 6, on cylinders): they are laid end to end in the segment's own columns, and
+// each lane counts the keys before its entries (equal keys are one lane's: their order there decides).
+template <int NMAX, int T>
+__device__ __forceinline__ int merge_lists(ColumnList<NMAX, T> &list, int N, int r, bool lane_ok, int lane, int gbase,
+                                           unsigned &mine, int &mine_h)
+{
+    __syncwarp();
+    int incl = list.n;
+    for (int off = 1; off < N; off <<= 1) {
+        const int t = __shfl_up_sync(kFull, incl, off);
+        if (r >= off) incl += t;
+    }
+    const int total = __shfl_sync(kFull, incl, lane_ok ? gbase + N - 1 : lane);
+    unsigned *seg = list.col - r;  // the segment's first column
+    // entry e of the segment: plane 2 NMAX + 2 (e / N), column e % N (its hit id on the next plane)
+    auto entry = [&](int e) {
+        const int q = e / N;
+        return (2 * NMAX + 2 * q) * T + e - q * N;
+    };
+    for (int i = 0; i < list.n; ++i) {
+        unsigned *d = seg + entry(incl - list.n + i);
+        d[0] = list.col[i * T];
+        d[T] = list.col[(NMAX + i) * T];
+    }
+    __syncwarp();
+    mine = kEmpty32;
+    mine_h = 0;
+    const int ns = lane_ok ? min(total, N) : 0;
+    if (lane_ok) {
+        for (int e = r; e < total; e += N) {
+            const unsigned *d = seg + entry(e);
+            const unsigned k = d[0];
+            int rank = 0;
+            for (int j = 0; j < total; ++j) rank += seg[entry(j)] < k + (unsigned)(j < e);
+            if (rank < N) {  // the lists are read: their first two planes take the winners
+                seg[rank] = k;
+                seg[T + rank] = d[T];
+            }
+        }
+    }
+    __syncwarp();
+    if (r < ns) {
+        mine = list.col[0];
+        mine_h = (int)list.col[T];
+    }
+    __syncwarp();
+    return ns;
 }
 
 // Hit ranges of phi sub-bins inside a bin, from the packed bytes of bin_sub (byte t - 1 holds
@@ -127,9 +248,9 @@ template <class R> __device__ __forceinline__ R asin_window(R x)
 // a.hit_dr off the cylinder (the two-step geometry of Sec. 2.2): the window around the
 // prediction on the average radius is widened by the track's travel over hit_dr, and each hit
 // inside it is scored after the second step to its own radius (step_chi2).
-template <int NMAX, class R, bool kTwo>
+template <class R, bool kTwo, class List>
 __device__ __forceinline__ void scan_window(const BuildArgs &a, int ev, int l, R Rl, const R p[6], const R P[21],
-                                            R chi2, int nh, int rank, unsigned (&lk)[NMAX], int (&lh)[NMAX])
+                                            R chi2, int nh, int rank, List &list)
 {
     const int seg = ev * a.L + l;
     const float2 vmax = a.var_max[seg];
@@ -232,13 +353,13 @@ __device__ __forceinline__ void scan_window(const BuildArgs &a, int ev, int l, R
                 else
                     c2 = chi2_uv<R>(P, u, v, sh, ch, R(hv.x), R(hv.y));
                 if (c2 < cut) {
-                    list_insert32(lk, lh, make_key32(nh + 1, to_f32(chi2 + c2), rank), __float_as_int(h.w));
+                    list.push(make_key32(nh + 1, to_f32(chi2 + c2), rank), __float_as_int(h.w));
                     found = true;
                 }
             }
         }
     }
-    if (!found) list_insert32(lk, lh, make_key32(nh, to_f32(chi2), rank), kHoleId);
+    if (!found) list.push(make_key32(nh, to_f32(chi2), rank), kHoleId);
 }
 
 // The same on an endcap disk (the "endcap z" of Sec. 2.2): the chi2-cut box |u| <= U (r-phi),
@@ -246,9 +367,9 @@ __device__ __forceinline__ void scan_window(const BuildArgs &a, int ev, int l, R
 // (r_h, phi_p + d) has u = r_p sin(d) and v = r_h - r_p cos(d): the box holds |d| <= asin(U / r_p)
 // and radii from r_p cos(asin(U / r_p)) - W to r_p + W, whose eta bins (eta = asinh(z / r) on the
 // disk at z) are scanned.  A compatible hit lies on the disk the state reached.
-template <int NMAX, class R>
+template <class R, class List>
 __device__ __forceinline__ void scan_window_disk(const BuildArgs &a, int ev, int l, const R p[6], const R P[21],
-                                                 R chi2, int nh, int rank, unsigned (&lk)[NMAX], int (&lh)[NMAX])
+                                                 R chi2, int nh, int rank, List &list)
 {
     const int seg = ev * a.L + l;
     const float2 vmax = a.var_max[seg];
@@ -322,13 +443,13 @@ __device__ __forceinline__ void scan_window_disk(const BuildArgs &a, int ev, int
                 if (ab(u) > U || ab(v) > W) continue;
                 const R c2 = chi2_disk<R>(p00, p10, p11, u, v, sh, ch, R(hv.x), R(hv.y));
                 if (c2 < cut) {
-                    list_insert32(lk, lh, make_key32(nh + 1, to_f32(chi2 + c2), rank), __float_as_int(h.w));
+                    list.push(make_key32(nh + 1, to_f32(chi2 + c2), rank), __float_as_int(h.w));
                     found = true;
                 }
             }
         }
     }
-    if (!found) list_insert32(lk, lh, make_key32(nh, to_f32(chi2), rank), kHoleId);
+    if (!found) list.push(make_key32(nh, to_f32(chi2), rank), kHoleId);
 }
 
 template <class R> __device__ __forceinline__ void store_track(void *par, void *cov, void *c2, int stride, int i,
@@ -470,7 +591,17 @@ __global__ void __launch_bounds__((BuildThreads<R, U>::value), (BuildMinBlocks<N
     static_assert((W & (W - 1)) == 0, "pooled updates rotate over a power-of-two number of warps");
     __shared__ int hist_hit[W][TKF_MAX_LAYERS][32];
     __shared__ signed char hist_par[W][TKF_MAX_LAYERS][32];
-    __shared__ float pool_st[kPool ? 32 * kThreads : 1];
+    // Lists of more than 6 branches go to shared memory: a lane rarely has more than three, and 20
+    // registers less leave the scan unspilled (N = 10, 20 events: 389 -> 357 us; two-step 3.29 -> 2.90
+    // ms for 183 k seeds; mixed 1.55 -> 1.38 ms).  Up to 6 they stay in registers (N = 6 in shared
+    // memory: 1.98 against 1.95 ms for 650 k seeds, N = 4 0.58 against 0.55 ms), and on endcap disks,
+    // whose windows hold more hits (N = 10: 1.48 against 1.20 ms).
+    constexpr bool kColumns = NMAX > 6 && !kDisk;
+    // planes of the branch lists (2 NMAX) and of their segments' lists (2 NMAX); the pooled updates park
+    // their states in the same ones, a thread in its own column
+    constexpr int kPlanes = kColumns ? 4 * NMAX : kPool ? 32 : 0;
+    __shared__ unsigned s_list[kPlanes > 0 ? kPlanes * kThreads : 1];
+    float *pool_st = (float *)s_list;
     __shared__ unsigned pool_bal[W];
     __shared__ int pool_tile;
     int pool_step = blockIdx.x;
@@ -544,50 +675,28 @@ __global__ void __launch_bounds__((BuildThreads<R, U>::value), (BuildMinBlocks<N
                 const R zd = pick<R>(a.disk_z_f[l], a.disk_z[l]);
                 const bool ok = alive && (disk ? propagate_plane<R>(p, P, p[2] >= R(0) ? zd : -zd, kb)
                                                : propagate<R>(p, P, Rl, kb));
-                unsigned lk[NMAX];
-                int lh[NMAX];
-#pragma unroll
-                for (int i = 0; i < NMAX; ++i) {
-                    lk[i] = kEmpty32;
-                    lh[i] = 0;
-                }
-                if (ok) {
-                    if (l == a.first && a.f_key) {
-                        // the first layer's window was scanned one lane per seed (k_first_scan)
-#pragma unroll
-                        for (int i = 0; i < NMAX; ++i) {
-                            lk[i] = __ldg(&a.f_key[(size_t)i * a.n_seeds + seed]);
-                            lh[i] = __ldg(&a.f_hit[(size_t)i * a.n_seeds + seed]);
-                        }
-                    } else if (disk) {
-                        scan_window_disk<NMAX, R>(a, ev, l, p, P, chi2, nh, r, lk, lh);
-                    } else {
-                        scan_window<NMAX, R, kTwo>(a, ev, l, Rl, p, P, chi2, nh, r, lk, lh);
-                    }
-                }
-
-                // merge the segment's lists: N rounds of a segmented minimum
                 unsigned mine = kEmpty32;
                 int mine_h = 0;
-                ns = 0;
-                for (int k = 0; k < N; ++k) {
-                    if (!__any_sync(kFull, lk[0] != kEmpty32)) break;  // no segment has branches left
-                    unsigned m = lk[0];
-                    for (int off = 1; off < N; off <<= 1) {
-                        const unsigned o = __shfl_down_sync(kFull, m, off);
-                        if (r + off < N && o < m) m = o;
+                if (l == a.first && a.f_key) {
+                    // the first layer's window was scanned one lane per seed (k_first_scan), into a
+                    // sorted list: the branch of rank r is its entry r
+                    const bool reached = __shfl_sync(kFull, (int)ok, lane_ok ? gbase : lane) != 0;
+                    if (has && reached) {
+                        mine = __ldg(&a.f_key[(size_t)r * a.n_seeds + seed]);
+                        mine_h = __ldg(&a.f_hit[(size_t)r * a.n_seeds + seed]);
                     }
-                    m = __shfl_sync(kFull, m, gbase);
-                    // the winner is the lane whose rank is the key's parent field
-                    const int hsel = __shfl_sync(kFull, lh[0], lane_ok ? gbase + (int)(m & 0xFu) : lane);
-                    if (m != kEmpty32) {
-                        if (lk[0] == m) list_pop32(lk, lh);
-                        if (r == k) {
-                            mine = m;
-                            mine_h = hsel;
-                        }
-                        ns = k + 1;
+                    const unsigned live = __ballot_sync(kFull, mine != kEmpty32);
+                    ns = lane_ok ? __popc((live >> gbase) & (kFull >> (32 - N))) : 0;
+                } else {
+                    using List = typename std::conditional<kColumns, ColumnList<NMAX, kThreads>, SortedList<NMAX>>::type;
+                    List list(s_list + threadIdx.x);
+                    if (ok) {
+                        if (disk)
+                            scan_window_disk<R>(a, ev, l, p, P, chi2, nh, r, list);
+                        else
+                            scan_window<R, kTwo>(a, ev, l, Rl, p, P, chi2, nh, r, list);
                     }
+                    ns = merge_lists(list, N, r, lane_ok, lane, gbase, mine, mine_h);
                 }
 
                 // survivors take their parent's predicted state
@@ -690,13 +799,7 @@ __global__ void __launch_bounds__(128) k_first_scan(const BuildArgs a)
     const int seed = blockIdx.x * blockDim.x + threadIdx.x;
     if (seed >= a.n_seeds) return;
     const int ev = a.s_event ? a.s_event[seed] : 0;
-    unsigned lk[NMAX];
-    int lh[NMAX];
-#pragma unroll
-    for (int i = 0; i < NMAX; ++i) {
-        lk[i] = kEmpty32;
-        lh[i] = 0;
-    }
+    SortedList<NMAX> list;
     if (ev >= 0 && ev < a.n_events) {  // k_build reports a bad event id
         R p[6], P[21];
         const R *sp = (const R *)a.s_par, *sc_ = (const R *)a.s_cov;
@@ -713,15 +816,15 @@ __global__ void __launch_bounds__(128) k_first_scan(const BuildArgs a)
         const bool ok = disk ? propagate_plane<R>(p, P, p[2] >= R(0) ? zd : -zd, kb) : propagate<R>(p, P, Rl, kb);
         if (ok) {
             if (disk)
-                scan_window_disk<NMAX, R>(a, ev, l, p, P, chi2, nh, 0, lk, lh);
+                scan_window_disk<R>(a, ev, l, p, P, chi2, nh, 0, list);
             else
-                scan_window<NMAX, R, kTwo>(a, ev, l, Rl, p, P, chi2, nh, 0, lk, lh);
+                scan_window<R, kTwo>(a, ev, l, Rl, p, P, chi2, nh, 0, list);
         }
     }
 #pragma unroll
     for (int i = 0; i < NMAX; ++i) {
-        a.f_key[(size_t)i * a.n_seeds + seed] = lk[i];
-        a.f_hit[(size_t)i * a.n_seeds + seed] = lh[i];
+        a.f_key[(size_t)i * a.n_seeds + seed] = list.lk[i];
+        a.f_hit[(size_t)i * a.n_seeds + seed] = list.lh[i];
     }
 }
 
