@@ -74,10 +74,12 @@ typedef struct {
     int32_t first_build_layer;        /* seeds are states on layer first_build_layer - 1 */
     int32_t precision;                /* enum tkf_precision */
     int32_t seeds_per_block;          /* seeds per work tile of the build kernel (one warp takes a
-                                         tile at a time); 0 = default */
+                                         tile at a time); 0 = as many as its lanes hold, fewer where
+                                         that would leave resident warps without a tile */
     int32_t seed_order;               /* 1: build seeds grouped by (event, eta bin, phi bin) so that a
-                                         warp's seeds share hit-index cache lines (results do not
-                                         depend on it); 0: in input order */
+                                         warp's seeds share hit-index cache lines, in batches large
+                                         enough for the grouping to pay (results do not depend on
+                                         it); 0: in input order */
     double hit_dr;                    /* cm, largest |hit radius - radius[layer]|.  0: hits lie on
                                          the cylinders.  > 0 (hits on modules off the average
                                          cylinder, the simplified CMS geometry of Sec. 2.2): fits

@@ -810,6 +810,8 @@ __global__ void k_seed_key(const IndexGeom g, int layer, const R *par, int strid
     atomicAdd(&counts[key], 1);
 }
 
+constexpr long long kOrderWork = 3'500'000;  // seeds times candidates from which tkf_build_tracks orders seeds
+
 __global__ void k_seed_place(const int *keys, int *counts, const int *off, int n, int *perm)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1692,9 +1694,6 @@ int tkf_build_tracks(tkf_ctx *ctx, const tkf_hit_index *idx, const tkf_tracks *s
     a.n_eta = c.n_eta_bins;
     a.n_phi = c.n_phi_bins;
     a.n_bins = c.n_eta_bins * c.n_phi_bins;
-    // default work tile: two groups of seeds per warp (small tiles keep every warp busy when
-    // a launch holds a single event)
-    a.seeds_per_block = c.seeds_per_block > 0 ? c.seeds_per_block : 2 * (32 / c.n_cand);
     a.n_seeds = seeds->n;
     a.n_events = idx->n_events;
     for (int l = 0; l < c.n_layers; ++l) {
@@ -1754,7 +1753,35 @@ int tkf_build_tracks(tkf_ctx *ctx, const tkf_hit_index *idx, const tkf_tracks *s
     a.tile_counter = ctx->d_tile;
     a.err = ctx->d_err;
     cudaStream_t s = (cudaStream_t)stream;
-    if (c.seed_order) {
+    const int nmax = build_nmax(c.n_cand);
+    auto launch = a.disk_mask    ? (c.precision == TKF_FP32    ? launch_build3_fp32
+                                    : c.precision == TKF_MIXED ? launch_build3_mixed
+                                                               : launch_build3_fp64)
+                  : c.hit_dr > 0.0 ? (c.precision == TKF_FP32    ? launch_build2_fp32
+                                    : c.precision == TKF_MIXED ? launch_build2_mixed
+                                                               : launch_build2_fp64)
+                                   : (c.precision == TKF_FP32    ? launch_build_fp32
+                                    : c.precision == TKF_MIXED ? launch_build_mixed
+                                                               : launch_build_fp64);
+    int occ = 0;
+    TKF_CUDA(ctx, launch(a, nmax, 0, nullptr, &occ));
+    const long long blocks = (long long)std::max(occ, 1) * ctx->sm_count;
+    // Default work tile: a warp's group of seeds, or fewer when the resident warps (4 a block) have not
+    // that many each -- a single event's seeds then run side by side instead of one group after
+    // another.  Two groups of five (before) / this: one event of 1000 seeds 124 / 109 us for its whole
+    // step (mixed, 3000 seeds: 194 / 153), 60 k seeds with N = 10 356 / 343 us, 245 k seeds with N = 4
+    // 549 / 530 us, 2.6 M seeds 8.93 / 8.95 ms.
+    const long long per_warp = (seeds->n + 4 * blocks - 1) / (4 * blocks);
+    a.seeds_per_block = c.seeds_per_block > 0
+                            ? c.seeds_per_block
+                            : (int)std::max<long long>(1, std::min<long long>(32 / c.n_cand, per_warp));
+    const long long tiles = ((long long)seeds->n + a.seeds_per_block - 1) / a.seeds_per_block;
+    const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, blocks));
+    // The ordering takes five launches (25 us and 0.03 us per thousand seeds) and makes the building
+    // 1 to 3 % faster: it pays from about 1.3 ms of building on.  With / without: 2.6 M seeds, N = 6,
+    // 8.95 / 9.05 ms for the step; 650 k seeds 1.938 / 1.937 ms; 245 k seeds, N = 4, 0.530 / 0.493 ms;
+    // 60 k seeds, N = 10, 0.343 / 0.310 ms; one event of 1000 seeds 108 / 92 us for the step.
+    if (c.seed_order && (long long)seeds->n * c.n_cand >= kOrderWork) {
         // counting sort of the seeds by (event, eta bin, phi bin) on the last seeding layer
         if ((st = tkf::seed_order_reserve(ctx, (size_t)seeds->n, (size_t)idx->n_events))) return st;
         const IndexGeom g = index_geom(c, idx->n_events);
@@ -1772,25 +1799,11 @@ int tkf_build_tracks(tkf_ctx *ctx, const tkf_hit_index *idx, const tkf_tracks *s
         k_seed_place<<<nb, 256, 0, s>>>(ctx->ord_key, ctx->ord_counts, ctx->ord_off, seeds->n, ctx->ord_perm);
         a.s_perm = ctx->ord_perm;  // counts are back to zero after k_seed_place
     }
-    const int nmax = build_nmax(c.n_cand);
     if (TKF_BUILD_FIRST_PASS && c.first_build_layer < c.n_layers && seeds->n > 0) {
         if ((st = tkf::first_list_reserve(ctx, (size_t)seeds->n))) return st;
         a.f_key = ctx->first_key;
         a.f_hit = ctx->first_hit;
     }
-    auto launch = a.disk_mask    ? (c.precision == TKF_FP32    ? launch_build3_fp32
-                                    : c.precision == TKF_MIXED ? launch_build3_mixed
-                                                               : launch_build3_fp64)
-                  : c.hit_dr > 0.0 ? (c.precision == TKF_FP32    ? launch_build2_fp32
-                                    : c.precision == TKF_MIXED ? launch_build2_mixed
-                                                               : launch_build2_fp64)
-                                   : (c.precision == TKF_FP32    ? launch_build_fp32
-                                    : c.precision == TKF_MIXED ? launch_build_mixed
-                                                               : launch_build_fp64);
-    int occ = 0;
-    TKF_CUDA(ctx, launch(a, nmax, 0, nullptr, &occ));
-    const long long tiles = ((long long)seeds->n + a.seeds_per_block - 1) / a.seeds_per_block;
-    const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, (long long)std::max(occ, 1) * ctx->sm_count));
     TKF_CUDA(ctx, cudaMemsetAsync(ctx->d_tile, 0, sizeof(int), s));
     TKF_CUDA(ctx, launch(a, nmax, grid, s, nullptr));
     TKF_CUDA(ctx, cudaGetLastError());
