@@ -126,7 +126,8 @@ struct tkf_ctx {
     size_t first_cap = 0;
     // seeding scratch: best layer-1 / layer-2 hit and score per first hit, first hits before each
     // event, the grids of layers 2 and 3 (SeedCells, cell tables, hits in cell order), seeds per
-    // compaction block and the tile queue
+    // compaction block and the tile queue; all in seed_mem
+    void *seed_mem = nullptr;
     int *seed_b = nullptr, *seed_c = nullptr, *seed_first = nullptr, *seed_tab = nullptr, *seed_id = nullptr,
         *seed_cnt = nullptr;
     float *seed_s = nullptr;

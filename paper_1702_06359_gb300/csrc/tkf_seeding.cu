@@ -844,9 +844,8 @@ int seed_cuda(tkf_ctx *ctx, cudaError_t e, const char *what)
 namespace tkf {
 void seed_scratch_free(tkf_ctx *ctx)
 {
-    for (void *p : {(void *)ctx->seed_b, (void *)ctx->seed_c, (void *)ctx->seed_s, ctx->seed_xyzr, (void *)ctx->seed_id,
-                    (void *)ctx->seed_first, ctx->seed_cells, (void *)ctx->seed_tab, (void *)ctx->seed_cnt})
-        cudaFree(p);
+    cudaFree(ctx->seed_mem);
+    ctx->seed_mem = nullptr;
     ctx->seed_b = ctx->seed_c = ctx->seed_id = ctx->seed_first = ctx->seed_tab = ctx->seed_cnt = nullptr;
     ctx->seed_s = nullptr;
     ctx->seed_xyzr = ctx->seed_cells = nullptr;
@@ -893,26 +892,41 @@ extern "C" int tkf_find_seeds(tkf_ctx *ctx, const tkf_hit_index *idx, const tkf_
     // every grid has at most kCellsPerHit cells per hit, kMinCells if that is more, and one entry more
     const size_t n_tab = std::min((size_t)kCellsPerHit * n + 2 * ne * (kMinCells + 1), 2 * ne * (kMaxCells + 1));
     if ((size_t)n > ctx->seed_cap || ne > ctx->seed_cap_events || n_tab > ctx->seed_cap_tab) {
+        // one allocation for all of it (each takes some ten microseconds of a first call)
+        const size_t cap = std::max<size_t>(std::max(n, 1), ctx->seed_cap), evs = std::max(ne, ctx->seed_cap_events),
+                     tab = std::max(n_tab, ctx->seed_cap_tab);
         seed_scratch_free(ctx);
-        const size_t cap = std::max(n, 1);
-        cudaError_t e;
-        if ((e = cudaMalloc(&ctx->seed_b, cap * sizeof(int))) != cudaSuccess ||
-            (e = cudaMalloc(&ctx->seed_c, cap * sizeof(int))) != cudaSuccess ||
-            (e = cudaMalloc(&ctx->seed_s, cap * sizeof(float))) != cudaSuccess ||
-            (e = cudaMalloc(&ctx->seed_xyzr, cap * sizeof(float4))) != cudaSuccess ||
-            (e = cudaMalloc(&ctx->seed_id, cap * sizeof(int))) != cudaSuccess ||
-            (e = cudaMalloc(&ctx->seed_first, (ne + 1) * sizeof(int))) != cudaSuccess ||
-            (e = cudaMalloc(&ctx->seed_cells, 2 * ne * sizeof(SeedCells))) != cudaSuccess ||
-            (e = cudaMalloc(&ctx->seed_tab, n_tab * sizeof(int))) != cudaSuccess ||
-            (e = cudaMalloc(&ctx->seed_cnt, (kCompactBlocks + 1) * sizeof(int))) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(k_seed_grid, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      kMaxCells * (int)sizeof(int))) != cudaSuccess) {
+        size_t bytes = 0;
+        auto part = [&](size_t count, size_t size) {
+            const size_t at = bytes;
+            bytes += (count * size + 255) / 256 * 256;
+            return at;
+        };
+        const size_t xyzr = part(cap, sizeof(float4)), cells = part(2 * evs, sizeof(SeedCells)),
+                     id = part(cap, sizeof(int)), res_b = part(cap, sizeof(int)), res_c = part(cap, sizeof(int)),
+                     res_s = part(cap, sizeof(float)), first = part(evs + 1, sizeof(int)),
+                     tabs = part(tab, sizeof(int)), cnt = part(kCompactBlocks + 1, sizeof(int));
+        cudaError_t e = cudaMalloc(&ctx->seed_mem, bytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_seed_grid, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kMaxCells * (int)sizeof(int));
+        if (e != cudaSuccess) {
             seed_scratch_free(ctx);
             return seed_cuda(ctx, e, "find_seeds: scratch");
         }
+        char *m = (char *)ctx->seed_mem;
+        ctx->seed_xyzr = m + xyzr;
+        ctx->seed_cells = m + cells;
+        ctx->seed_id = (int *)(m + id);
+        ctx->seed_b = (int *)(m + res_b);
+        ctx->seed_c = (int *)(m + res_c);
+        ctx->seed_s = (float *)(m + res_s);
+        ctx->seed_first = (int *)(m + first);
+        ctx->seed_tab = (int *)(m + tabs);
+        ctx->seed_cnt = (int *)(m + cnt);
         ctx->seed_cap = cap;
-        ctx->seed_cap_events = ne;
-        ctx->seed_cap_tab = n_tab;
+        ctx->seed_cap_events = evs;
+        ctx->seed_cap_tab = tab;
     }
     if (n == 0) {
         cudaError_t e = cudaMemsetAsync(n_found, 0, sizeof(int32_t), s);
