@@ -1804,7 +1804,8 @@ int tkf_build_tracks(tkf_ctx *ctx, const tkf_hit_index *idx, const tkf_tracks *s
         a.f_key = ctx->first_key;
         a.f_hit = ctx->first_hit;
     }
-    TKF_CUDA(ctx, cudaMemsetAsync(ctx->d_tile, 0, sizeof(int), s));
+    // (k_first_scan, where there is one, resets the tile counter)
+    if (!a.f_key) TKF_CUDA(ctx, cudaMemsetAsync(ctx->d_tile, 0, sizeof(int), s));
     TKF_CUDA(ctx, launch(a, nmax, grid, s, nullptr));
     TKF_CUDA(ctx, cudaGetLastError());
     return TKF_OK;

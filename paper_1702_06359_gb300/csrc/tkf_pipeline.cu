@@ -71,7 +71,8 @@ struct tkf_pipeline {
     tkf_hit_index *idx = nullptr;
     Buf seeds, built, final_, back;
     double back_scale = 0.0;  // > 0: the step ends with the backward pass (covariance scale)
-    cudaStream_t capture = nullptr;
+    cudaStream_t capture = nullptr, side = nullptr;  // of the capture: the sequence, and its branch
+    cudaEvent_t fork = nullptr, join = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     Signature sig{};
@@ -96,12 +97,20 @@ int issue(tkf_pipeline *p, const tkf_hits *hits, const int32_t *seed_hits, const
 {
     tkf_ctx *ctx = p->ctx;
     const int L = ctx->cfg.n_layers, first = ctx->cfg.first_build_layer, stride = p->max_tracks;
-    int st = tkf_build_hit_index(ctx, hits, &p->idx, (tkf_stream)s);
-    if (st) return st;
     tkf_tracks seeds = view(p->seeds, n, stride), built = view(p->built, n, stride),
                fin = view(p->final_, n, stride);
     seeds.event = const_cast<int32_t *>(seed_event);
-    if ((st = tkf::seed_and_fit(ctx, hits, seed_hits, first - 1, &seeds, (tkf_stream)s))) return st;
+    // The seed fit reads hits by their input position, not the index: in a graph the two are branches
+    // side by side (neither fills the chip: one event of 1000 tracks 92.7 us for the step in sequence, 88.0
+    // so and without the tile counter's memset; 3000 tracks 114.9 and 107.2, 640 events 8.91 and 8.89 ms).
+    // A step issued kernel by kernel keeps one stream: the four calls of a branch cost the host as much.
+    const cudaStream_t seed_stream = capturing ? p->side : s;
+    if (capturing && (cudaEventRecord(p->fork, s) != cudaSuccess || cudaStreamWaitEvent(p->side, p->fork, 0) != cudaSuccess))
+        return fail(ctx, TKF_ERR_CUDA, "pipeline: fork");
+    int st = tkf::seed_and_fit(ctx, hits, seed_hits, first - 1, &seeds, (tkf_stream)seed_stream);
+    if (st || (st = tkf_build_hit_index(ctx, hits, &p->idx, (tkf_stream)s))) return st;
+    if (capturing && (cudaEventRecord(p->join, p->side) != cudaSuccess || cudaStreamWaitEvent(s, p->join, 0) != cudaSuccess))
+        return fail(ctx, TKF_ERR_CUDA, "pipeline: join");
     // events around the building kernel (event-record nodes when captured into the graph)
     const unsigned flag = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (cudaEventRecordWithFlags(p->build_ev[0], s, flag) != cudaSuccess)
@@ -140,6 +149,9 @@ int tkf_pipeline_create(tkf_ctx *ctx, int32_t max_hits, int32_t max_events, int3
     for (Buf *b : {&p->seeds, &p->built, &p->final_})
         if (e == cudaSuccess) e = alloc_buf(*b, max_tracks, L, es);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->capture, cudaStreamNonBlocking);
+    if (e == cudaSuccess && p->use_graph) e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking);
+    if (e == cudaSuccess && p->use_graph) e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
+    if (e == cudaSuccess && p->use_graph) e = cudaEventCreateWithFlags(&p->join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreate(&p->build_ev[0]);
     if (e == cudaSuccess) e = cudaEventCreate(&p->build_ev[1]);
     int st = e == cudaSuccess ? TKF_OK : (e == cudaErrorMemoryAllocation ? TKF_ERR_NOMEM : TKF_ERR_CUDA);
@@ -159,8 +171,9 @@ int tkf_pipeline_destroy(tkf_pipeline *p)
     if (!p) return TKF_ERR_INVALID;
     if (p->exec) cudaGraphExecDestroy(p->exec);
     if (p->graph) cudaGraphDestroy(p->graph);
-    if (p->capture) cudaStreamDestroy(p->capture);
-    for (cudaEvent_t ev : p->build_ev)
+    for (cudaStream_t st : {p->capture, p->side})
+        if (st) cudaStreamDestroy(st);
+    for (cudaEvent_t ev : {p->build_ev[0], p->build_ev[1], p->fork, p->join})
         if (ev) cudaEventDestroy(ev);
     if (p->idx) tkf_hit_index_free(p->idx);
     for (Buf *b : {&p->seeds, &p->built, &p->final_, &p->back}) free_buf(*b);
