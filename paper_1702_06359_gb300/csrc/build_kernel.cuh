@@ -585,6 +585,7 @@ template <int NMAX, class R, class U, bool kTwo, bool kExactN, bool kDisk>
 __global__ void __launch_bounds__((BuildThreads<R, U>::value), (BuildMinBlocks<NMAX, R, U, kTwo, kExactN, kDisk>::value))
     k_build(const BuildArgs a)
 {
+    after_previous();
     constexpr int kThreads = BuildThreads<R, U>::value;
     constexpr int W = kThreads / 32;
     constexpr bool kPool = BuildThreads<R, U>::pool;
@@ -797,6 +798,8 @@ template <int NMAX, class R, bool kTwo, bool kDisk>
 __global__ void __launch_bounds__(128) k_first_scan(const BuildArgs a)
 {
     const int seed = blockIdx.x * blockDim.x + threadIdx.x;
+    after_previous();
+    allow_next();
     if (seed == 0) *a.tile_counter = 0;  // k_build's (a memset of its own took 1.5 us of a small event's step)
     if (seed >= a.n_seeds) return;
     const int ev = a.s_event ? a.s_event[seed] : 0;
@@ -849,7 +852,9 @@ cudaError_t launch_build_t(const BuildArgs &a, int nmax, int grid, cudaStream_t 
 #undef TKF_K
     constexpr int threads = BuildThreads<R, U>::value;
     if (occupancy) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, fn, threads, 0);
-    void *args[] = {(void *)&a};
+    auto go = [&](const void *f, int blocks, int th) {
+        return launch_next((void (*)(BuildArgs))f, (unsigned)blocks, (unsigned)th, 0, s, a);
+    };
     if (a.f_key && a.first < a.L && a.n_seeds > 0) {
         const void *ff = nullptr;
 #define TKF_F(n) (const void *)k_first_scan<n, R, kTwo, kDisk>
@@ -861,10 +866,10 @@ cudaError_t launch_build_t(const BuildArgs &a, int nmax, int grid, cudaStream_t 
         default: ff = TKF_F(16); break;
         }
 #undef TKF_F
-        const cudaError_t e = cudaLaunchKernel(ff, dim3((a.n_seeds + 127) / 128), dim3(128), args, 0, s);
+        const cudaError_t e = go(ff, (a.n_seeds + 127) / 128, 128);
         if (e != cudaSuccess) return e;
     }
-    return cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, 0, s);
+    return go(fn, grid, threads);
 }
 
 }  // namespace tkf

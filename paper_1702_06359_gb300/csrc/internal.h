@@ -102,6 +102,36 @@ int first_list_reserve(tkf_ctx *ctx, size_t max_seeds);
 // Frees the seeding scratch of a context.
 void seed_scratch_free(tkf_ctx *ctx);
 
+// A kernel that may be set up while the one before it in its stream still runs (programmatic dependent
+// launch): every thread of it starts with after_previous(), which waits until that one and all it
+// waited for are complete and their writes visible.  Where the one before calls allow_next() at its start the
+// blocks are placed as soon as its own all run, otherwise when they have ended; a long kernel (k_build,
+// k_seed_find) does not call it, so that no waiting block holds an SM that another stream could use.
+// What the kernel before writes is read by plain loads: the compiler may move loads of the
+// non-coherent path (const __restrict__, __ldg) up past the wait within a basic block.
+// Before / with it: 20 events' index 57.3 / 53.2 us, one event's step 87.8 / 84.5, seeds of a small
+// event 82.5 / 73.9, 60 k seeds built with N = 10 309 / 301, the server's 12 events 750 / 739, 640 events
+// 8.93 / 8.93 ms.
+template <class... P, class... A>
+cudaError_t launch_next(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, P(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
 inline int build_nmax(int n)
 {
     return n <= 1 ? 1 : n <= 4 ? 4 : n <= 6 ? 6 : n <= 10 ? 10 : 16;

@@ -459,6 +459,8 @@ __global__ void __launch_bounds__(kLayerThreads) k_index_layers(const IndexGeom 
                                                                 int *seg_count, int *seg_runs, int *seg_start, int *err)
 {
     __shared__ int s_cnt[TKF_MAX_LAYERS], s_runs[TKF_MAX_LAYERS], s_start[TKF_MAX_LAYERS];
+    after_previous();
+    allow_next();
     const int e = blockIdx.x, tid = threadIdx.x;
     const int h0 = h.event_off[e], h1 = h.event_off[e + 1];
     if (tid < g.L) s_cnt[tid] = s_runs[tid] = s_start[tid] = 0;
@@ -569,12 +571,13 @@ template <int T, class F> __device__ __forceinline__ void for_hits(const tkf_hit
 // 0.73 ms.
 template <int T, int kPerSM, bool kLast>
 __global__ void __launch_bounds__(T, kPerSM)
-k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int *__restrict__ seg_count,
-                const int *__restrict__ seg_runs, const int *__restrict__ seg_start, int lo, int cap, float4 *hxyzi,
-                float2 *hvar, uint4 *bin_sub, int *pos_of_hit, int *bin_off, float2 *var_max)
+k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int *seg_count, const int *seg_runs,
+                const int *seg_start, int lo, int cap, float4 *hxyzi, float2 *hvar, uint4 *bin_sub, int *pos_of_hit, int *bin_off, float2 *var_max)
 {
     extern __shared__ uint4 s_words[];
     __shared__ int s_part[T / 32], s_mu, s_mv;
+    after_previous();
+    allow_next();
     const unsigned full = 0xffffffffu;
     const int seg = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int cnt = seg_count[seg];
@@ -764,17 +767,19 @@ cudaError_t launch_segment_index(const IndexGeom &g, const tkf_hits &h, int sm_c
 {
     const unsigned n_segs = (unsigned)(g.n_events * g.L);
     int *cnt = seg, *runs = seg + n_segs, *start = runs + n_segs;
-    k_index_layers<<<(unsigned)g.n_events, kLayerThreads, 0, s>>>(g, h, ev_off, cnt, runs, start, err);
+    cudaError_t e = launch_next(k_index_layers, (unsigned)g.n_events, kLayerThreads, 0, s, g, h, ev_off, cnt, runs, start,
+                                err);
     int lo = -1;
     auto take = [&](auto kern, int threads, size_t smem) {
         const int hi = segment_cap(g.n_bins, smem);
-        kern<<<n_segs, threads, smem, s>>>(g, h, cnt, runs, start, lo, hi, hxyzi, hvar, bin_sub, pos_of_hit, bin_off,
-                                           var_max);
+        if (e == cudaSuccess)
+            e = launch_next(kern, n_segs, threads, smem, s, g, h, cnt, runs, start, lo, hi, hxyzi, hvar, bin_sub,
+                            pos_of_hit, bin_off, var_max);
         lo = std::max(hi, -1);
     };
     if ((int)n_segs > sm_count) take(k_index_segment<kSegThreads, 2, false>, kSegThreads, kSegSmem);
     take(k_index_segment<kSegThreadsBig, 1, true>, kSegThreadsBig, kSegSmemBig);
-    return cudaGetLastError();
+    return e;
 }
 
 // Allows the segment kernels their dynamic shared memory on the current device.
@@ -920,6 +925,8 @@ __device__ __forceinline__ void seed_estimate(const FitGeom &g, const tkf_hits &
 template <class R>
 __global__ void k_seed(const FitGeom g, const tkf_hits h, const int *seed_hits, tkf_tracks out, int *err)
 {
+    after_previous();
+    allow_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= out.n) return;
     const int h1 = seed_hits[i], h2 = seed_hits[out.stride + i], h3 = seed_hits[2 * out.stride + i];
@@ -1048,6 +1055,8 @@ template <class R, class U, bool kDisk>
 __global__ void __launch_bounds__(kFitThreads, (FitMinBlocks<R, U>::value)) k_fit(const FitGeom g, const tkf_hits h, const tkf_tracks in, const int *hit_idx, int first, int last,
                       int prop_first, tkf_tracks out, int *err)
 {
+    after_previous();
+    allow_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= in.n) return;
     const size_t si = in.stride, so = out.stride;
@@ -1072,6 +1081,8 @@ __global__ void __launch_bounds__(kFitThreads, (FitMinBlocks<R, U>::value)) k_fi
 template <class R, class U, bool kDisk>
 __global__ void __launch_bounds__(kFitThreads, (FitMinBlocks<R, U>::value)) k_seed_fit(const FitGeom g, const tkf_hits h, const int *seed_hits, int last, tkf_tracks out, int *err)
 {
+    after_previous();
+    allow_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= out.n) return;
     const size_t st = out.stride;
@@ -1124,6 +1135,8 @@ template <class R, class U, bool kDisk>
 __global__ void __launch_bounds__(kFitThreads, (FitMinBlocks<R, U>::value)) k_fit_backward(const FitGeom g, const tkf_hits h, const tkf_tracks in, const int *hit_idx, int last,
                                int first, R scale, tkf_tracks out, int *err)
 {
+    after_previous();
+    allow_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= in.n) return;
     const size_t si = in.stride, so = out.stride;
@@ -1599,7 +1612,8 @@ int tkf::fit_tracks(tkf_ctx *ctx, const tkf_hits *hits, const tkf_tracks *init, 
     cudaStream_t s = (cudaStream_t)stream;
     const int pf = continue_fit ? 1 : 0;
     auto go = [&](auto kern) {
-        kern<<<(nn + th - 1) / th, th, 0, s>>>(g, *hits, *init, hidx, first_layer, last_layer, pf, *out, ctx->d_err);
+        (void)launch_next(kern, (nn + th - 1) / th, th, 0, s, g, *hits, *init, hidx, first_layer, last_layer, pf, *out,
+                          ctx->d_err);  // an error stays for cudaGetLastError
     };
     const bool dk = g.disk_mask != 0;
     switch (ctx->cfg.precision) {
@@ -1629,7 +1643,8 @@ int tkf::fit_backward(tkf_ctx *ctx, const tkf_hits *hits, const tkf_tracks *init
     const int nn = init->n, th = ctx->cfg.precision == TKF_FP64 ? kFitThreadsF64 : kFitThreads;
     cudaStream_t s = (cudaStream_t)stream;
     auto go = [&](auto kern, auto scale) {
-        kern<<<(nn + th - 1) / th, th, 0, s>>>(g, *hits, *init, hidx, last_layer, first_layer, scale, *out, ctx->d_err);
+        (void)launch_next(kern, (nn + th - 1) / th, th, 0, s, g, *hits, *init, hidx, last_layer, first_layer, scale, *out,
+                          ctx->d_err);
     };
     const bool dk = g.disk_mask != 0;
     const float sf = (float)cov_scale;
@@ -1659,7 +1674,9 @@ int tkf::seed_and_fit(tkf_ctx *ctx, const tkf_hits *hits, const int32_t *seed_hi
     const FitGeom g = fit_geom(ctx);
     const int nn = out->n, th = ctx->cfg.precision == TKF_FP64 ? kFitThreadsF64 : kFitThreads;
     cudaStream_t s = (cudaStream_t)stream;
-    auto go = [&](auto kern) { kern<<<(nn + th - 1) / th, th, 0, s>>>(g, *hits, seed_hits, last_layer, *out, ctx->d_err); };
+    auto go = [&](auto kern) {
+        (void)launch_next(kern, (nn + th - 1) / th, th, 0, s, g, *hits, seed_hits, last_layer, *out, ctx->d_err);
+    };
     const bool dk = g.disk_mask != 0;
     switch (ctx->cfg.precision) {
     case TKF_FP32: dk ? go(k_seed_fit<float, float, true>) : go(k_seed_fit<float, float, false>); break;

@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(1024) k_seed_plan(const SeedGeom g, const int 
     __shared__ int s_a[32], s_b[32];
     __shared__ int carry_a, carry_b;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    allow_next();
     if (tid == 0) carry_a = carry_b = *queue = 0;
     __syncthreads();
     for (int base = 0; base < g.n_events; base += blockDim.x) {
@@ -224,6 +225,7 @@ __global__ void __launch_bounds__(kGridThreads, 1)
 k_seed_grid(const SeedGeom g, const float4 *__restrict__ hxyzi, const int *__restrict__ bin_off, SeedCells *cells,
             int *__restrict__ tab, float4 *__restrict__ gxyzr, int *__restrict__ gid)
 {
+    after_previous();
     extern __shared__ int s_cnt[];
     __shared__ float s_lo[32], s_hi[32];
     __shared__ int s_part[32];
@@ -783,6 +785,8 @@ __device__ __forceinline__ int block_sum(int v, int *s_part)
 
 __global__ void __launch_bounds__(kSeedThreads) k_seed_count(const int *res_b, const int *n_first, int *count)
 {
+    after_previous();
+    allow_next();
     __shared__ int s_part[kSeedThreads / 32];
     const int2 c = chunk_of(*n_first);
     int v = 0;
@@ -796,6 +800,7 @@ k_seed_scatter(const SeedGeom g, const float4 *hxyzi, const int *bin_off, const 
                const int *res_b, const int *res_c, const float *res_s, const int *count, int max_seeds, int *seed_hits,
                int *seed_event, float *seed_score, int *total)
 {
+    after_previous();
     __shared__ int s_part[kSeedThreads / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int before = 0;
@@ -962,8 +967,8 @@ extern "C" int tkf_find_seeds(tkf_ctx *ctx, const tkf_hit_index *idx, const tkf_
     float4 *xyzr = (float4 *)ctx->seed_xyzr;
     int *queue = ctx->seed_cnt + kCompactBlocks;
     k_seed_plan<<<1, 1024, 0, s>>>(g, idx->bin_off, ctx->seed_first, cells, queue);
-    k_seed_grid<<<dim3((unsigned)ne, 2), kGridThreads, grid_cells(n) * sizeof(int), s>>>(
-        g, idx->hxyzi, idx->bin_off, cells, ctx->seed_tab, xyzr, ctx->seed_id);
+    cudaError_t e = launch_next(k_seed_grid, dim3((unsigned)ne, 2), kGridThreads, grid_cells(n) * sizeof(int), s, g,
+                                idx->hxyzi, idx->bin_off, cells, ctx->seed_tab, xyzr, ctx->seed_id);
     // Lanes per first hit, by the tiles of 32 first hits (a layer holds about n / L hits) for each
     // warp the GPU holds.  Measured with 1 / 2 / 4 / 8 lanes: 36 tiles a warp 7.00 / 7.08 / 8.09 /
     // 10.1 ms, 9 tiles 1.86 / 1.83 / 2.04 / 2.52 ms, 0.9 tiles 507 / 306 / 288 / 308 us, a sixth of a
@@ -983,10 +988,12 @@ extern "C" int tkf_find_seeds(tkf_ctx *ctx, const tkf_hit_index *idx, const tkf_
         find(k_seed_find<4>);
     else
         find(k_seed_find<8>);
-    k_seed_count<<<kCompactBlocks, kSeedThreads, 0, s>>>(ctx->seed_b, ctx->seed_first + ne, ctx->seed_cnt);
-    k_seed_scatter<<<kCompactBlocks, kSeedThreads, 0, s>>>(g, idx->hxyzi, idx->bin_off, idx->ev_off, ctx->seed_first,
-                                                           ctx->seed_b, ctx->seed_c, ctx->seed_s, ctx->seed_cnt,
-                                                           max_seeds, seed_hits, seed_event, seed_score, n_found);
-    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = launch_next(k_seed_count, kCompactBlocks, kSeedThreads, 0, s, ctx->seed_b, ctx->seed_first + ne, ctx->seed_cnt);
+    if (e == cudaSuccess)
+        e = launch_next(k_seed_scatter, kCompactBlocks, kSeedThreads, 0, s, g, idx->hxyzi, idx->bin_off, idx->ev_off,
+                        ctx->seed_first, ctx->seed_b, ctx->seed_c, ctx->seed_s, ctx->seed_cnt, max_seeds, seed_hits,
+                        seed_event, seed_score, n_found);
+    if (e == cudaSuccess) e = cudaGetLastError();
     return e == cudaSuccess ? TKF_OK : seed_cuda(ctx, e, "find_seeds: launch");
 }
