@@ -104,13 +104,16 @@ void seed_scratch_free(tkf_ctx *ctx);
 
 // A kernel that may be set up while the one before it in its stream still runs (programmatic dependent
 // launch): every thread of it starts with after_previous(), which waits until that one and all it
-// waited for are complete and their writes visible.  Where the one before calls allow_next() at its start the
-// blocks are placed as soon as its own all run, otherwise when they have ended; a long kernel (k_build,
-// k_seed_find) does not call it, so that no waiting block holds an SM that another stream could use.
+// waited for are complete and their writes visible.  Its blocks are placed when those of the one before have
+// ended, or, where that one calls allow_next() at its start, as soon as its blocks all run.  That pays
+// before a kernel of few blocks (k_first_scan before k_build: one event's step 88.9 / 84.7 us; between the
+// seeding's kernels 75.1 / 73.8).  Blocks placed early go where a slot is free, not where the work is
+// least: the double fits lost by it (40 k tracks both ways 1115 -> 1305 us), the index's second size class
+// too (512 events 710 -> 720), and a long kernel's successors would hold slots that another stream could use.
 // What the kernel before writes is read by plain loads: the compiler may move loads of the
 // non-coherent path (const __restrict__, __ldg) up past the wait within a basic block.
-// Before / with it: 20 events' index 57.3 / 53.2 us, one event's step 87.8 / 84.5, seeds of a small
-// event 82.5 / 73.9, 60 k seeds built with N = 10 309 / 301, the server's 12 events 750 / 739, 640 events
+// Plain launches / these: 20 events' index 57.3 / 52, one event's step 87.8 / 84.5, seeds of a small
+// event 82.5 / 73.8, 60 k seeds built with N = 10 309 / 300, the server's 12 events 750 / 735, 640 events
 // 8.93 / 8.93 ms.
 template <class... P, class... A>
 cudaError_t launch_next(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, A &&...args)

@@ -460,7 +460,6 @@ __global__ void __launch_bounds__(kLayerThreads) k_index_layers(const IndexGeom 
 {
     __shared__ int s_cnt[TKF_MAX_LAYERS], s_runs[TKF_MAX_LAYERS], s_start[TKF_MAX_LAYERS];
     after_previous();
-    allow_next();
     const int e = blockIdx.x, tid = threadIdx.x;
     const int h0 = h.event_off[e], h1 = h.event_off[e + 1];
     if (tid < g.L) s_cnt[tid] = s_runs[tid] = s_start[tid] = 0;
@@ -577,7 +576,6 @@ k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int
     extern __shared__ uint4 s_words[];
     __shared__ int s_part[T / 32], s_mu, s_mv;
     after_previous();
-    allow_next();
     const unsigned full = 0xffffffffu;
     const int seg = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int cnt = seg_count[seg];
@@ -926,7 +924,6 @@ template <class R>
 __global__ void k_seed(const FitGeom g, const tkf_hits h, const int *seed_hits, tkf_tracks out, int *err)
 {
     after_previous();
-    allow_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= out.n) return;
     const int h1 = seed_hits[i], h2 = seed_hits[out.stride + i], h3 = seed_hits[2 * out.stride + i];
@@ -1056,7 +1053,6 @@ __global__ void __launch_bounds__(kFitThreads, (FitMinBlocks<R, U>::value)) k_fi
                       int prop_first, tkf_tracks out, int *err)
 {
     after_previous();
-    allow_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= in.n) return;
     const size_t si = in.stride, so = out.stride;
@@ -1082,7 +1078,6 @@ template <class R, class U, bool kDisk>
 __global__ void __launch_bounds__(kFitThreads, (FitMinBlocks<R, U>::value)) k_seed_fit(const FitGeom g, const tkf_hits h, const int *seed_hits, int last, tkf_tracks out, int *err)
 {
     after_previous();
-    allow_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= out.n) return;
     const size_t st = out.stride;
@@ -1136,7 +1131,6 @@ __global__ void __launch_bounds__(kFitThreads, (FitMinBlocks<R, U>::value)) k_fi
                                int first, R scale, tkf_tracks out, int *err)
 {
     after_previous();
-    allow_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= in.n) return;
     const size_t si = in.stride, so = out.stride;
