@@ -44,10 +44,9 @@ FLOP_WINDOW = 40       # chi2 bounding box -> eta/phi bin ranges
 FLOP_CHI2 = 39         # one hit: tangent-plane residual, 2x2 S, chi2, half-cylinder test
 FLOP_UPDATE = 335      # Kalman gain, state update, Joseph-form covariance
 FLOP_SCATTER = 30      # Highland width and the four covariance terms
-# FP64 operations of one MIXED Kalman update (kalman_update<double, float>): B = H P (18), S and
-# its determinant (11), the inverse's three terms (3), chi2 (9), gain (36), D = B^T - K S (48),
-# Joseph form (168); conversions and the division are not counted
-FLOP_UPDATE_FP64 = 290
+# FP32 instructions of one MIXED Kalman update (mixed_update: the double update's 290 operations on
+# pairs of floats), counted as one operation each
+FLOP_UPDATE_PAIRS = 900
 # Work per seed on the batched workload, counted with the oracle's instrumentation
 # (python oracle/opcount.py --events 16 --workload batched, 53756 seeds):
 PER_SEED = dict(n_prop=19.2502, n_hits_examined=189.7167, n_updates=18.0985, n_kept=21.7897)
@@ -77,36 +76,36 @@ MODULE_DR = 1.0  # cm between the inner and outer module rows of a layer (hit_dr
 FLOP_PROPAGATE_PLANE, FLOP_WINDOW_DISK, FLOP_CHI2_DISK, FLOP_UPDATE_DISK, FLOP_SCATTER_DISK = 296, 57, 57, 359, 23
 PER_SEED_DISK = dict(n_prop=25.7421, n_hits_examined=218.2409, n_updates=26.9508, n_kept=29.2005)
 # DRAM bytes (read + write) per seed of the FP32 endcap building (k_first_scan + k_build; one ncu
-# capture of its 640-event launches: 130.8 + 480.2 MB for 649 624 seeds; summary in profiles/);
+# capture of its 640-event launches: 130.9 + 483.9 MB for 649 624 seeds; summary in profiles/);
 # None when a kernel changes
-BUILD3_DRAM_BYTES_PER_SEED = 940.6
+BUILD3_DRAM_BYTES_PER_SEED = 946.4
 FLOP_PER_SEED_DISK = (PER_SEED_DISK["n_prop"] * (FLOP_PROPAGATE_PLANE + FLOP_WINDOW_DISK)
                       + PER_SEED_DISK["n_hits_examined"] * FLOP_CHI2_DISK
                       + PER_SEED_DISK["n_updates"] * FLOP_UPDATE_DISK
                       + PER_SEED_DISK["n_kept"] * 6.0 / 7.0 * FLOP_SCATTER_DISK)
 # DRAM bytes (read + write) per seed of the two-step FP32 building (k_first_scan + k_build), from
-# one ncu capture of the kernels as built now (160-event case: 124.2 + 434.8 MB for 701 095
+# one ncu capture of the kernels as built now (160-event case: 124.3 + 435.4 MB for 701 095
 # seeds; summary in profiles/); None whenever a kernel changes until it is captured again
-BUILD2_DRAM_BYTES_PER_SEED = 797.3
+BUILD2_DRAM_BYTES_PER_SEED = 798.4
 # Warp instructions per seed of the building kernels (ncu smsp__inst_executed.sum of the same
-# captures: 47.3 M + 1.675 G one-step, 170.9 M + 3.516 G two-step, for 701 095 seeds), for the
+# captures: 46.5 M + 1.544 G one-step, 168.6 M + 3.394 G two-step, for 701 095 seeds), for the
 # instruction-issue roofline beside the FP32 one: an SM sub-partition issues at most one warp
 # instruction per cycle, 4 per SM; None whenever a kernel changes until it is captured again
-BUILD_WARP_INST_PER_SEED, BUILD2_WARP_INST_PER_SEED = 2455.9, 5259.1
+BUILD_WARP_INST_PER_SEED, BUILD2_WARP_INST_PER_SEED = 2268.2, 5082.0
 # FP32 FMA peak of a GB300: 152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz (maximum SM clock)
 SM_COUNT, FP32_LANES, SM_MAX_GHZ = 152, 128, 2.07
-# libtkf.so kernels per step: hit index (event order, per-event count/scan/place, bin sort),
+# libtkf.so kernels per step: hit index (hits per layer, segments in two size classes),
 # seed estimate with seed fit, seed ordering (key, segment totals, segment scan, bin scan,
 # place), first-layer scan, build, final fit
 KERNELS_PER_STEP = 12
 # DRAM bytes (read + write) per seed of the FP32 building (k_first_scan + k_build), from one ncu
-# capture of the kernels as built now (160-event case: 124.1 + 433.3 MB for 701 095 seeds;
+# capture of the kernels as built now (160-event case: 123.1 + 435.2 MB for 701 095 seeds;
 # summary in profiles/); None whenever a kernel changes until it is captured again
-BUILD_DRAM_BYTES_PER_SEED = 795.1
+BUILD_DRAM_BYTES_PER_SEED = 796.4
 # warp instructions of k_seed_find per layer-0 hit and active lanes per instruction, from one ncu
-# capture of the 160-event seeding case (3.185 G instructions for 932 025 first hits; summary in
+# capture of the 160-event seeding case (1.195 G instructions for 932 025 first hits; summary in
 # profiles/); None whenever the kernel changes until it is captured again
-SEED_WARP_INST_PER_FIRST_HIT, SEED_LANES_ACTIVE = 3417.5, 19.01
+SEED_WARP_INST_PER_FIRST_HIT, SEED_LANES_ACTIVE = 1281.7, 26.56
 FP32_PEAK_TFLOPS = SM_COUNT * FP32_LANES * 2 * SM_MAX_GHZ / 1e3
 ISSUE_PEAK_WARP_INST_PER_S = SM_COUNT * 4 * SM_MAX_GHZ * 1e9
 
@@ -1015,7 +1014,7 @@ def main():
             "tracks": b4.n_tracks, "hits": b4.n_hits, "first_layer_hits": n_first, "seeds": n_found,
             "seeds_per_track": n_found / b4.n_tracks, "own_triplet": own_trip,
             "roofline": None if SEED_WARP_INST_PER_FIRST_HIT is None else {
-                "kernel": "k_seed_find (+ k_seed_count, k_seed_scan, k_seed_scatter in seeding_ms)", "bound": "issue",
+                "kernel": "k_seed_find (+ k_seed_plan, k_seed_grid, k_seed_count, k_seed_scatter in seeding_ms)", "bound": "issue",
                 "achieved": SEED_WARP_INST_PER_FIRST_HIT * n_first / (seed_ms / 1e3),
                 "peak": ISSUE_PEAK_WARP_INST_PER_S, "unit": "warp instructions/s",
                 "frac": SEED_WARP_INST_PER_FIRST_HIT * n_first / (seed_ms / 1e3) / ISSUE_PEAK_WARP_INST_PER_S,
@@ -1026,8 +1025,8 @@ def main():
             "cuts": {k: getattr(cuts4, k) for k in ("pt_min", "kappa_slack", "z_vertex", "d0_max", "dz_max",
                                                     "conf_rphi", "conf_z", "confirm")},
             "form": "the batched workload's events 0..%d with pixel resolution (20 um r-phi, 50 um z) on layers "
-                    "0-3: tkf_find_seeds over the hit index (k_seed_find, one thread per layer-0 hit, then "
-                    "count, scan and scatter) timed alone (seeding_ms); value = simulated tracks per second "
+                    "0-3: tkf_find_seeds over the hit index (grids of layers 2 and 3, k_seed_find, "
+                    "then count and scatter) timed alone (seeding_ms); value = simulated tracks per second "
                     "of the chain hit index + seeding + pipeline (its own index, seed fit, building, final "
                     "fit) with the found seeds; FP32, N = 6" % (b4.n_events - 1)}
         p4.close()
@@ -1121,23 +1120,20 @@ def main():
         mctx.sync_status(stream)
         mms = m0.elapsed_time(m1) / a.steps
         mb_ms = statistics.mean(mb)
-        m_fp64 = PER_SEED["n_updates"] * FLOP_UPDATE_FP64 * n_tr / (mb_ms / 1e3) / 1e12
+        m_flop = FLOP_PER_SEED + PER_SEED["n_updates"] * (FLOP_UPDATE_PAIRS - FLOP_UPDATE)
+        m_tflops = m_flop * n_tr / (mb_ms / 1e3) / 1e12
         mixed = {"value": n_tr / (mms / 1e3), "unit": UNIT, "ms_per_step": mms, "build_ms": mb_ms,
-                 "roofline": {"kernel": "k_first_scan + k_build<6,float,double>", "bound": "fp64", "achieved": m_fp64,
-                              "peak": None, "unit": "TFLOP/s", "frac": None,
-                              "flop_per_seed_fp64": PER_SEED["n_updates"] * FLOP_UPDATE_FP64,
-                              "note": "FP64 arithmetic of the updates against the measured FP64 multiply-add "
-                                      "rate (alu_peaks); each block's updates run packed into full warps; ncu "
-                                      "shows the FP64 pipe 77 % busy at 19 of 32 active lanes, the rest of its "
-                                      "work the update's other double operations (reciprocal, negations, "
-                                      "compares)"},
-                 "precision": "mixed: FP32 propagation, window and chi2; FP64 innovation inverse and Joseph update",
+                 "roofline": {"kernel": "k_first_scan + k_build<6,float,double>", "bound": "alu", "achieved": m_tflops,
+                              "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": m_tflops / FP32_PEAK_TFLOPS,
+                              "flop_per_seed": m_flop,
+                              "note": "the FP32 form's operations, with the updates' double arithmetic on pairs of "
+                                      "floats (one operation per instruction); each block's updates run packed into "
+                                      "full warps"},
+                 "precision": "mixed: FP32 propagation, window and chi2; innovation inverse and Joseph update on pairs "
+                              "of floats (48 bits)",
                  "seeds_per_warp_tile": best_tile}
         mpipe.close()
         mctx.close()
-        if alu is not None:
-            mixed["roofline"]["peak"] = alu["fp64_tflops"]
-            mixed["roofline"]["frac"] = m_fp64 / alu["fp64_tflops"]
 
     # ---------------- plain form: one event per pass (direct launches), per-event latency
     plain = None
