@@ -38,6 +38,8 @@ namespace tkf {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr unsigned kEmpty32 = 0xFFFFFFFFu;
+constexpr int kFirstThreads = 128;                 // of k_first_scan's blocks
+constexpr int kFirstWide = kFirstThreads * 152;  // seeds from which such blocks reach every SM
 
 template <class R> __device__ __forceinline__ R pick(float f, double d);
 template <> __device__ __forceinline__ float pick<float>(float f, double) { return f; }
@@ -791,7 +793,7 @@ __global__ void __launch_bounds__((BuildThreads<R, U>::value), (BuildMinBlocks<N
 // 29 scattered words per seed left this kernel waiting on memory), and an event's seeds still
 // come together, so its hits stay in L2.
 template <int NMAX, class R, bool kTwo, bool kDisk>
-__global__ void __launch_bounds__(128) k_first_scan(const BuildArgs a)
+__global__ void __launch_bounds__(kFirstThreads) k_first_scan(const BuildArgs a)
 {
     const int seed = blockIdx.x * blockDim.x + threadIdx.x;
     after_previous();
@@ -862,7 +864,10 @@ cudaError_t launch_build_t(const BuildArgs &a, int nmax, int grid, cudaStream_t 
         default: ff = TKF_F(16); break;
         }
 #undef TKF_F
-        const cudaError_t e = go(ff, (a.n_seeds + 127) / 128, 128);
+        // blocks of one warp where blocks of four would leave SMs without one: an event of 1000 tracks 82.9 ->
+        // 78.4 us for its step, of 3000 and 5000 the same; 2.6 M seeds 8.371 ms with 128 threads, 8.383 with 32
+        const int fth = a.n_seeds < kFirstWide ? 32 : kFirstThreads;
+        const cudaError_t e = go(ff, (a.n_seeds + fth - 1) / fth, fth);
         if (e != cudaSuccess) return e;
     }
     return go(fn, grid, threads);

@@ -48,7 +48,7 @@ class Chain:
 
 
 @pytest.mark.parametrize("precision", [tkf.FP32, tkf.MIXED, tkf.FP64], ids=["fp32", "mixed", "fp64"])
-@pytest.mark.parametrize("events,tracks", [(1, 40), (3, 900), (40, 250)])
+@pytest.mark.parametrize("events,tracks", [(1, 33), (1, 1000), (3, 900), (40, 250), (20, 1024)])
 def test_a_chain_of_calls_gives_what_single_calls_give(events, tracks, precision):
     b = generate(EventSpec(seed=17, n_events=events, n_tracks=tracks, noise_frac=0.4), Detector())
     chain = Chain(b, precision)
