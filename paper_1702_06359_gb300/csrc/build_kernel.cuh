@@ -681,8 +681,8 @@ __global__ void __launch_bounds__((BuildThreads<R, U>::value), (BuildMinBlocks<N
                     // sorted list: the branch of rank r is its entry r
                     const bool reached = __shfl_sync(kFull, (int)ok, lane_ok ? gbase : lane) != 0;
                     if (has && reached) {
-                        mine = __ldg(&a.f_key[(size_t)r * a.n_seeds + seed]);
-                        mine_h = __ldg(&a.f_hit[(size_t)r * a.n_seeds + seed]);
+                        mine = a.f_key[(size_t)r * a.n_seeds + seed];  // written by the kernel before: plain loads
+                        mine_h = a.f_hit[(size_t)r * a.n_seeds + seed];
                     }
                     const unsigned live = __ballot_sync(kFull, mine != kEmpty32);
                     ns = lane_ok ? __popc((live >> gbase) & (kFull >> (32 - N))) : 0;
