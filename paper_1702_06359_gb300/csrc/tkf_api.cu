@@ -1,6 +1,7 @@
 // libtkf.so: context, hit index, seed estimate and track fit kernels, and the C ABI entry
 // points declared in include/tkf.h.
 #include <cuda_runtime.h>
+#include <math_constants.h>
 
 #include <algorithm>
 #include <cmath>
@@ -739,6 +740,14 @@ k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int
             mv = fmaxf(mv, vv);
         }
     }
+    // Hits whose layer is out of range have no bin, and the event's segments start at its first position, so
+    // as many positions stay free behind its last segment, inside the range of its last bin.  They take
+    // hits that no window holds (its tests are comparisons, which fail on NaN).
+    if (l == g.L - 1)
+        for (int pos = base + cnt + tid, end = h.event_off[e + 1]; pos < end; pos += T) {
+            hxyzi[pos] = make_float4(CUDART_NAN_F, CUDART_NAN_F, CUDART_NAN_F, __int_as_float(0));
+            hvar[pos] = make_float2(0.f, 0.f);
+        }
     // the largest variances (the order of non-negative floats is that of their bits)
     const unsigned ru = __reduce_max_sync(full, __float_as_uint(mu)), rv = __reduce_max_sync(full, __float_as_uint(mv));
     if (lane == 0) {
