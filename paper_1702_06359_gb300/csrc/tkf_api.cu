@@ -679,7 +679,12 @@ k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int
         for_hits<T>(h, i0, cnt, place);
     } else {
         int *s_bin = (int *)s_words;  // counts, then cursors: start of a bin, then its end
-        unsigned *g_ord = (unsigned *)(hvar + base);  // order word (sixteenth, id) q at 2 q
+        // order word q: sixteenth and id, the id whole (an event over the hit limit, which is reported, has ids
+        // beyond 23 bits; two words that compared equal would leave a position of the index unwritten)
+        unsigned long long *g_ord = (unsigned long long *)(hvar + base);
+        auto order_word = [&](unsigned key, int i) {
+            return ((unsigned long long)(key & (kSubBins - 1)) << 32) | (unsigned)(i - h0);
+        };
         for (int b = tid; b < g.n_bins; b += T) s_bin[b] = 0;
         __syncthreads();
         for (int i = i0 + tid; i < i1; i += T) {
@@ -711,22 +716,21 @@ k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int
         for (int i = i0 + tid; i < i1; i += T) {
             if (h.layer[i] != l) continue;
             const unsigned key = (unsigned)pos_of_hit[i];
-            g_ord[2 * (size_t)atomicAdd(&s_bin[key / kSubBins], 1)] =
-                ((key & (kSubBins - 1)) << 23) | ((unsigned)(i - h0) & 0x7FFFFFu);
+            g_ord[atomicAdd(&s_bin[key / kSubBins], 1)] = order_word(key, i);
         }
         __syncthreads();
         for (int b = tid; b < g.n_bins; b += T) {
             const int a0 = b ? s_bin[b - 1] : 0, a1 = s_bin[b];
             bin_off[b0 + b] = base + a0;
-            bin_sub[b0 + b] = sub_starts([&](int t) { return (int)g_ord[2 * (size_t)t]; }, a0, a1);
+            bin_sub[b0 + b] = sub_starts([&](int t) { return (int)(g_ord[t] >> 32) << 23; }, a0, a1);
         }
         for (int i = i0 + tid; i < i1; i += T) {
             if (h.layer[i] != l) continue;
             const unsigned key = (unsigned)pos_of_hit[i], b = key / kSubBins;
-            const unsigned word = ((key & (kSubBins - 1)) << 23) | ((unsigned)(i - h0) & 0x7FFFFFu);
+            const unsigned long long word = order_word(key, i);
             const int a0 = b ? s_bin[b - 1] : 0, a1 = s_bin[b];
             int pos = base + a0;
-            for (int t = a0; t < a1; ++t) pos += g_ord[2 * (size_t)t] < word;
+            for (int t = a0; t < a1; ++t) pos += g_ord[t] < word;
             pos_of_hit[i] = pos;
         }
         __syncthreads();  // every word has been compared: hvar takes the variances

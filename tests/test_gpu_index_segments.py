@@ -119,3 +119,36 @@ def test_a_dense_bin_and_many_equal_sixteenths():
     rng = np.random.default_rng(3)
     layer = np.repeat(np.arange(L), 3000)
     _check(*_hits(rng, layer, width=0.03), layer, np.array([0, len(layer)], dtype=np.int32))
+
+
+@pytest.mark.parametrize("order", ["grouped", "random"])
+def test_an_event_over_the_hit_limit_fills_its_part_of_the_index(order):
+    """2^23 + 5 hits of one event among enough small ones for k_index_segment; the last five lie where the
+    first five do, so that they share their sixteenths with ids equal to theirs in the lowest 23 bits."""
+    rng = np.random.default_rng(8)
+    big, small = (1 << 23) + 5, 40
+    n_ev = 60  # 16384 hits per segment on average would be 9.8 M
+    layer = rng.integers(0, L, big)
+    if order == "grouped":
+        layer = np.sort(layer)
+    layer[-5:] = layer[:5]
+    layer = np.concatenate([layer, np.tile(np.arange(small) // 4, n_ev - 1)])
+    off = np.concatenate([[0], big + small * np.arange(n_ev)]).astype(np.int32)
+    x, y, z = _hits(rng, layer)
+    for a in (x, y, z):
+        a[big - 5:big] = a[:5]
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda")  # noqa: E731
+    n = len(layer)
+    v = torch.full((n,), 1e-4, device="cuda")
+    ctx = tkf.Context()
+    idx = ctx.build_hit_index(tkf.DeviceHits(t(x), t(y), t(z), v, v, t(layer.astype(np.int32)), t(off)))
+    with pytest.raises(tkf.TkfError, match="8388606"):
+        ctx.sync_status()
+    w = idx.view()
+    pos, xyzi = _view(w.pos_of_hit, (n,), "<i4"), _view(w.hit_xyzi, (n, 4), "<f4")
+    assert np.array_equal(np.sort(pos), np.arange(n))
+    ev = np.repeat(np.arange(n_ev), np.diff(off))
+    assert np.array_equal(xyzi[pos, :3], np.stack([x, y, z], 1))
+    assert np.array_equal(xyzi[pos, 3].view(np.int32), np.arange(n) - off[ev])
+    idx.free()
+    ctx.close()
