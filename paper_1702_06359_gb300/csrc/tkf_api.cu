@@ -452,19 +452,34 @@ k_bin_sort(const IndexGeom g, const int *bin_off, const int *ev_off, int n_bins_
 // every hit straight to its place.  Positions are read twice (the second time from L2), variances
 // once, everything else is written once: 52 bytes a hit from and to HBM where counting, placing and
 // ordering in separate kernels moved 124.
+//
+// Where the hits of a layer do not follow one another in the input, its block first lists them
+// (list_layer), reading the event's layers twice more, from L2.  Events with their hits in a random
+// order, with the lists / by the multi-launch kernels above: one of 13 k hits 22 / 45 us, of 65 k 57 / 64 us,
+// of 160 k 120 / 102 us (ten blocks, each fetching 32 bytes for 4), 20 of 67 k 102 / 192 us, 160 of 55 k on
+// average 0.64 / 1.05 ms.  Passing over the hits of other layers instead: 41, 188, 506, 380 us, 2.25 ms.
 
-// Hits of each (event, layer): count, runs of consecutive hits on the layer, and the first hit of
-// (any) one of them; one block per event.  Copies the event offsets into the index.
+// The layers of hits i .. i + 3 (-1 outside h0 .. h1 - 1), as one word where the array is aligned to it.
+__device__ __forceinline__ int4 layer_word(const tkf_hits &h, bool aligned, int i, int h0, int h1)
+{
+    if (aligned && i >= h0 && i + 4 <= h1) return __ldg((const int4 *)(h.layer + i));
+    auto one = [&](int k) { return k >= h0 && k < h1 ? __ldg(&h.layer[k]) : -1; };
+    return make_int4(one(i), one(i + 1), one(i + 2), one(i + 3));
+}
+
+// Hits of each (event, layer) and the first of them (-1: they do not follow one another), one block per
+// event; copies the event offsets into the index.
 constexpr int kLayerThreads = 1024;
 __global__ void __launch_bounds__(kLayerThreads) k_index_layers(const IndexGeom g, const tkf_hits h, int *ev_off,
-                                                                int *seg_count, int *seg_runs, int *seg_start, int *err)
+                                                                int *seg_count, int *seg_start, int *err)
 {
-    __shared__ int s_cnt[TKF_MAX_LAYERS], s_runs[TKF_MAX_LAYERS], s_start[TKF_MAX_LAYERS];
+    __shared__ int s_cnt[TKF_MAX_LAYERS], s_runs[TKF_MAX_LAYERS], s_start[TKF_MAX_LAYERS], s_mixed;
     after_previous();
     const int e = blockIdx.x, tid = threadIdx.x;
     const int h0 = h.event_off[e], h1 = h.event_off[e + 1];
     if (tid < g.L) s_cnt[tid] = s_runs[tid] = s_start[tid] = 0;
     if (tid == 0) {
+        s_mixed = 0;
         ev_off[e] = h0;
         if (e == g.n_events - 1) ev_off[e + 1] = h1;
         if (h1 - h0 > kMaxHitsPerEvent) atomicOr(err, kErrTooManyHits);  // 23-bit local ids
@@ -474,7 +489,7 @@ __global__ void __launch_bounds__(kLayerThreads) k_index_layers(const IndexGeom 
     // words in flight (the largest event's block is the kernel's tail)
     const bool aligned = ((size_t)h.layer & 15) == 0;
     constexpr int U = 4;
-    for (int p0 = (h0 & ~3) + 4 * tid; p0 < h1; p0 += U * 4 * kLayerThreads) {
+    for (int p0 = (h0 & ~3) + 4 * tid; p0 < h1 && !*(volatile int *)&s_mixed; p0 += U * 4 * kLayerThreads) {
         int l[U][6];  // layers of hits i0 - 1 .. i0 + 4
 #pragma unroll
         for (int v = 0; v < U; ++v) {
@@ -499,6 +514,12 @@ __global__ void __launch_bounds__(kLayerThreads) k_index_layers(const IndexGeom 
             if (i0 > h0 && i0 + 4 < h1 && l[v][0] == l[v][1] && l[v][1] == l[v][2] && l[v][2] == l[v][3] &&
                 l[v][3] == l[v][4] && l[v][4] == l[v][5] && l[v][1] >= 0 && l[v][1] < g.L)
                 continue;
+            // three runs that start in one word: the layers are mixed, and counted below
+            if (i0 >= h0 && i0 + 4 <= h1 &&
+                (l[v][0] != l[v][1]) + (l[v][1] != l[v][2]) + (l[v][2] != l[v][3]) + (l[v][3] != l[v][4]) >= 3) {
+                s_mixed = 1;
+                continue;
+            }
 #pragma unroll
             for (int u = 1; u < 5; ++u) {
                 const int i = i0 + u - 1, c = l[v][u];
@@ -517,9 +538,56 @@ __global__ void __launch_bounds__(kLayerThreads) k_index_layers(const IndexGeom 
         }
     }
     __syncthreads();
+    bool mixed = s_mixed;
+    for (int l = 0; l < g.L; ++l) mixed |= s_runs[l] > 1;
+    if (mixed) {  // block-uniform: count hit by hit, a thread's in bytes
+        static_assert(TKF_MAX_LAYERS == 16, "a byte of c for each layer");
+        __syncthreads();
+        if (tid < g.L) {
+            s_cnt[tid] = 0;
+            s_start[tid] = -1;
+        }
+        __syncthreads();
+        unsigned c[4] = {0, 0, 0, 0};
+        auto count = [&](int i, int l) {
+            if (i < h0 || i >= h1) return;
+            if (l < 0 || l >= g.L) {
+                atomicOr(err, kErrBadLayer);
+                return;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) c[k] += l >> 2 == k ? 1u << (8 * (l & 3)) : 0u;
+        };
+        int held = 0;  // hits a byte may hold
+        for (int q0 = h0 & ~3; q0 < h1; q0 += U * 4 * kLayerThreads) {  // every thread takes every turn
+            int4 q[U];
+#pragma unroll
+            for (int v = 0; v < U; ++v) q[v] = layer_word(h, aligned, q0 + 4 * (tid + v * kLayerThreads), h0, h1);
+#pragma unroll
+            for (int v = 0; v < U; ++v) {
+                const int i = q0 + 4 * (tid + v * kLayerThreads);
+                count(i, q[v].x);
+                count(i + 1, q[v].y);
+                count(i + 2, q[v].z);
+                count(i + 3, q[v].w);
+            }
+            held += 4 * U;
+            if (held + 4 * U > 255 || q0 + U * 4 * kLayerThreads >= h1) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {  // the warp's sums fit 16 bits
+                    const unsigned even = __reduce_add_sync(0xffffffffu, c[k] & 0x00FF00FFu),
+                                   odd = __reduce_add_sync(0xffffffffu, c[k] >> 8 & 0x00FF00FFu);
+                    if ((tid & 31) < 4 && 4 * k + (tid & 3) < g.L)
+                        atomicAdd(&s_cnt[4 * k + (tid & 3)], (int)((tid & 1 ? odd : even) >> (tid & 2 ? 16 : 0) & 0xFFFFu));
+                    c[k] = 0;
+                }
+                held = 0;
+            }
+        }
+        __syncthreads();
+    }
     if (tid < g.L) {
         seg_count[e * g.L + tid] = s_cnt[tid];
-        seg_runs[e * g.L + tid] = s_runs[tid];
         seg_start[e * g.L + tid] = s_start[tid];
     }
 }
@@ -535,16 +603,58 @@ int segment_cap(int n_bins, size_t smem) { return ((int)smem - 16 * seg_words(n_
 
 __device__ __forceinline__ unsigned half16(const unsigned *w, unsigned k) { return (w[k >> 1] >> (16 * (k & 1))) & 0xFFFFu; }
 
+// Lists the hits of layer l among an event's h0 .. h1 - 1 (all of the block): each warp counts and then
+// places those of a stretch of the event.  s_part: a word per warp.
+template <int T>
+__device__ __noinline__ void list_layer(const tkf_hits &h, int l, int h0, int h1, int *list, int *s_part)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const bool aligned = ((size_t)h.layer & 15) == 0;
+    const int q0 = h0 & ~3, n = (h1 - q0 + 3) / 4, per = (n + T - 1) / T * 32;  // words, words a warp
+    const int a = min(w * per, n), b = min(a + per, n);
+    constexpr int U = 4;
+    auto each = [&](auto f) {  // f(first hit of this lane's word, its layers)
+        for (int q = a; q < b; q += 32 * U) {
+            int4 v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int k = q + 32 * u + lane;
+                v[u] = k < b ? layer_word(h, aligned, q0 + 4 * k, h0, h1) : make_int4(-1, -1, -1, -1);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) f(q0 + 4 * (q + 32 * u + lane), v[u]);
+        }
+    };
+    int cnt = 0;
+    each([&](int, int4 v) { cnt += (v.x == l) + (v.y == l) + (v.z == l) + (v.w == l); });
+    cnt = __reduce_add_sync(full, cnt);
+    if (lane == 0) s_part[w] = cnt;
+    __syncthreads();
+    for (int k = 0; k < w; ++k) list += s_part[k];
+    each([&](int i, int4 v) {
+        const unsigned x = __ballot_sync(full, v.x == l), y = __ballot_sync(full, v.y == l),
+                       z = __ballot_sync(full, v.z == l), t = __ballot_sync(full, v.w == l), below = (1u << lane) - 1u;
+        int *p = list + __popc(x & below) + __popc(y & below) + __popc(z & below) + __popc(t & below);
+        if (v.x == l) *p++ = i;
+        if (v.y == l) *p++ = i + 1;
+        if (v.z == l) *p++ = i + 2;
+        if (v.w == l) *p = i + 3;
+        list += __popc(x) + __popc(y) + __popc(z) + __popc(t);
+    });
+    __syncthreads();  // (s_part is free again)
+}
+
 // One pass of a segment's hits through its block: f(position in the segment, x, y, z), U hits per thread
-// loaded together.
-template <int T, class F> __device__ __forceinline__ void for_hits(const tkf_hits &h, int i0, int cnt, F f)
+// loaded together; at(j): the id of its hit j.
+template <int T, class A, class F> __device__ __forceinline__ void for_hits(const tkf_hits &h, A at, int cnt, F f)
 {
     constexpr int U = 4;
     for (int j0 = threadIdx.x; j0 < cnt; j0 += U * T) {
         float x[U], y[U], z[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int i = i0 + min(j0 + u * T, cnt - 1);
+            const int i = at(min(j0 + u * T, cnt - 1));
             x[u] = h.x[i];
             y[u] = h.y[i];
             z[u] = h.z[i];
@@ -555,11 +665,9 @@ template <int T, class F> __device__ __forceinline__ void for_hits(const tkf_hit
     }
 }
 
-// The segment of one (event, layer).  A launch takes the segments of one run with lo < hits <= cap,
-// held in shared memory; the last launch (kLast) also those that are larger or whose hits are not
-// consecutive: only their bins are counted there, the hits' keys live in pos_of_hit and their order
-// words in hvar until the final positions are known, and hits on other layers in between are passed
-// over.
+// The segment of one (event, layer).  A launch takes the segments with lo < hits <= cap, held in shared
+// memory; the last launch (kLast) also the larger ones: only their bins are counted there, the
+// hits' keys live in pos_of_hit and their order words in hvar until the final positions are known.
 //
 // What bounds it: the latency of its phases (loads, counting, scan, tables, placing, each behind a
 // barrier) with 73 % of the warps resident and 40 % issue; 512 events (23.5 M hits) move 1.7 GB in 0.70
@@ -571,8 +679,8 @@ template <int T, class F> __device__ __forceinline__ void for_hits(const tkf_hit
 // 0.73 ms.
 template <int T, int kPerSM, bool kLast>
 __global__ void __launch_bounds__(T, kPerSM)
-k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int *seg_count, const int *seg_runs,
-                const int *seg_start, int lo, int cap, float4 *hxyzi, float2 *hvar, uint4 *bin_sub, int *pos_of_hit, int *bin_off, float2 *var_max)
+k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int *seg_count,
+                const int *seg_start, int *list, int lo, int cap, float4 *hxyzi, float2 *hvar, uint4 *bin_sub, int *pos_of_hit, int *bin_off, float2 *var_max)
 {
     extern __shared__ uint4 s_words[];
     __shared__ int s_part[T / 32], s_mu, s_mv;
@@ -580,13 +688,21 @@ k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int
     const unsigned full = 0xffffffffu;
     const int seg = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int cnt = seg_count[seg];
-    const bool grouped = seg_runs[seg] <= 1, fast = grouped && cnt <= cap && cnt < 65536;
+    const bool fast = cnt <= cap && cnt < 65536;
     if (fast ? cnt <= lo : !kLast) return;
     const int e = seg / g.L, l = seg - e * g.L;
     const int h0 = h.event_off[e];
     int base = h0;
     for (int k = 0; k < l; ++k) base += seg_count[e * g.L + k];
-    const int i0 = grouped ? seg_start[seg] : h0, i1 = grouped ? i0 + cnt : h.event_off[e + 1];
+    const int start = seg_start[seg];
+    if (start < 0) list_layer<T>(h, l, h0, h.event_off[e + 1], list + base, s_part);
+    // the segment's hits in the order of their ids: consecutive, or listed
+    auto each_way = [&](auto f) {
+        if (start < 0)
+            f([=](int j) { return list[base + j]; });
+        else
+            f([=](int j) { return start + j; });
+    };
     const float rl = g.radius[l];
     const bool disk = (g.disk_mask >> l) & 1u;
     const size_t b0 = (size_t)seg * g.n_bins;
@@ -600,10 +716,12 @@ k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int
         for (int k = tid; k < nw; k += T) s_words[k] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
         // (1) the sixteenth of every hit; hits per sixteenth
-        for_hits<T>(h, i0, cnt, [&](int j, float x, float y, float z) {
-            const unsigned key = hit_key(g, rl, disk, x, y, z);
-            s_key[j] = (unsigned short)key;
-            atomicAdd(&s_cell[key >> 1], key & 1 ? 0x10000u : 1u);
+        each_way([&](auto at) {
+            for_hits<T>(h, at, cnt, [&](int j, float x, float y, float z) {
+                const unsigned key = hit_key(g, rl, disk, x, y, z);
+                s_key[j] = (unsigned short)key;
+                atomicAdd(&s_cell[key >> 1], key & 1 ? 0x10000u : 1u);
+            });
         });
         __syncthreads();
         // (2) inclusive scan: the end of every sixteenth; thread t owns a contiguous chunk of words, an
@@ -662,21 +780,22 @@ k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int
             bin_sub[b0 + b] = sub;
         }
         // (5) the hits to their places: a sixteenth's hits in the order of their ids
-        auto place = [&](int j, float x, float y, float z) {
-            const unsigned key = s_key[j];
-            const int a0 = (int)half16(s_cell, key), a1 = (int)half16(s_cell, key + 1);
-            int pos = base + a0;
-            if (a1 - a0 > 1)
-                for (int t = a0; t < a1; ++t) pos += s_ord[t] < j;
-            const int i = i0 + j;
-            const float vu = h.var_u[i], vv = h.var_v[i];
-            hxyzi[pos] = make_float4(x, y, z, __int_as_float(i - h0));
-            hvar[pos] = make_float2(vu, vv);
-            pos_of_hit[i] = pos;
-            mu = fmaxf(mu, vu);
-            mv = fmaxf(mv, vv);
-        };
-        for_hits<T>(h, i0, cnt, place);
+        each_way([&](auto at) {
+            for_hits<T>(h, at, cnt, [&](int j, float x, float y, float z) {
+                const unsigned key = s_key[j];
+                const int a0 = (int)half16(s_cell, key), a1 = (int)half16(s_cell, key + 1);
+                int pos = base + a0;
+                if (a1 - a0 > 1)
+                    for (int t = a0; t < a1; ++t) pos += s_ord[t] < j;
+                const int i = at(j);
+                const float vu = h.var_u[i], vv = h.var_v[i];
+                hxyzi[pos] = make_float4(x, y, z, __int_as_float(i - h0));
+                hvar[pos] = make_float2(vu, vv);
+                pos_of_hit[i] = pos;
+                mu = fmaxf(mu, vu);
+                mv = fmaxf(mv, vv);
+            });
+        });
     } else {
         int *s_bin = (int *)s_words;  // counts, then cursors: start of a bin, then its end
         // order word q: sixteenth and id, the id whole (an event over the hit limit, which is reported, has ids
@@ -687,8 +806,8 @@ k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int
         };
         for (int b = tid; b < g.n_bins; b += T) s_bin[b] = 0;
         __syncthreads();
-        for (int i = i0 + tid; i < i1; i += T) {
-            if (h.layer[i] != l) continue;
+        for (int j = tid; j < cnt; j += T) {
+            const int i = start < 0 ? list[base + j] : start + j;
             const unsigned key = hit_key(g, rl, disk, h.x[i], h.y[i], h.z[i]);
             pos_of_hit[i] = (int)key;
             atomicAdd(&s_bin[key / kSubBins], 1);
@@ -713,8 +832,8 @@ k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int
             run += c;
         }
         __syncthreads();
-        for (int i = i0 + tid; i < i1; i += T) {
-            if (h.layer[i] != l) continue;
+        for (int j = tid; j < cnt; j += T) {
+            const int i = start < 0 ? list[base + j] : start + j;
             const unsigned key = (unsigned)pos_of_hit[i];
             g_ord[atomicAdd(&s_bin[key / kSubBins], 1)] = order_word(key, i);
         }
@@ -724,8 +843,8 @@ k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int
             bin_off[b0 + b] = base + a0;
             bin_sub[b0 + b] = sub_starts([&](int t) { return (int)(g_ord[t] >> 32) << 23; }, a0, a1);
         }
-        for (int i = i0 + tid; i < i1; i += T) {
-            if (h.layer[i] != l) continue;
+        for (int j = tid; j < cnt; j += T) {
+            const int i = start < 0 ? list[base + j] : start + j;
             const unsigned key = (unsigned)pos_of_hit[i], b = key / kSubBins;
             const unsigned long long word = order_word(key, i);
             const int a0 = b ? s_bin[b - 1] : 0, a1 = s_bin[b];
@@ -734,8 +853,8 @@ k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int
             pos_of_hit[i] = pos;
         }
         __syncthreads();  // every word has been compared: hvar takes the variances
-        for (int i = i0 + tid; i < i1; i += T) {
-            if (h.layer[i] != l) continue;
+        for (int j = tid; j < cnt; j += T) {
+            const int i = start < 0 ? list[base + j] : start + j;
             const int pos = pos_of_hit[i];
             const float vu = h.var_u[i], vv = h.var_v[i];
             hxyzi[pos] = make_float4(h.x[i], h.y[i], h.z[i], __int_as_float(i - h0));
@@ -771,20 +890,19 @@ bool segment_index(int n_hits, size_t n_segs, int n_bins)
     return n_bins <= kSegMaxBins && n_bins >= 4 && (size_t)n_hits <= n_segs * 16384;
 }
 
-// seg: 3 n_segs words of scratch.
-cudaError_t launch_segment_index(const IndexGeom &g, const tkf_hits &h, int sm_count, int *seg, int *ev_off,
+// seg: 2 n_segs words of scratch; list: one word for each hit.
+cudaError_t launch_segment_index(const IndexGeom &g, const tkf_hits &h, int sm_count, int *seg, int *list, int *ev_off,
                                  float4 *hxyzi, float2 *hvar, uint4 *bin_sub, int *pos_of_hit, int *bin_off,
                                  float2 *var_max, int *err, cudaStream_t s)
 {
     const unsigned n_segs = (unsigned)(g.n_events * g.L);
-    int *cnt = seg, *runs = seg + n_segs, *start = runs + n_segs;
-    cudaError_t e = launch_next(k_index_layers, (unsigned)g.n_events, kLayerThreads, 0, s, g, h, ev_off, cnt, runs, start,
-                                err);
+    int *cnt = seg, *start = seg + n_segs;
+    cudaError_t e = launch_next(k_index_layers, (unsigned)g.n_events, kLayerThreads, 0, s, g, h, ev_off, cnt, start, err);
     int lo = -1;
     auto take = [&](auto kern, int threads, size_t smem) {
         const int hi = segment_cap(g.n_bins, smem);
         if (e == cudaSuccess)
-            e = launch_next(kern, n_segs, threads, smem, s, g, h, cnt, runs, start, lo, hi, hxyzi, hvar, bin_sub,
+            e = launch_next(kern, n_segs, threads, smem, s, g, h, cnt, start, list, lo, hi, hxyzi, hvar, bin_sub,
                             pos_of_hit, bin_off, var_max);
         lo = std::max(hi, -1);
     };
@@ -1486,7 +1604,7 @@ int tkf_build_hit_index(tkf_ctx *ctx, const tkf_hits *hits, tkf_hit_index **out,
         cudaStream_t s = (cudaStream_t)stream;
         const IndexGeom g = index_geom(c, hits->n_events);
         if (segment_index(hits->n, n_segs, NB)) {
-            TKF_CUDA(ctx, launch_segment_index(g, *hits, ctx->sm_count, idx->counts, idx->ev_off, idx->hxyzi, idx->hvar,
+            TKF_CUDA(ctx, launch_segment_index(g, *hits, ctx->sm_count, idx->counts, idx->keys, idx->ev_off, idx->hxyzi, idx->hvar,
                                                idx->bin_sub, idx->pos_of_hit, idx->bin_off, idx->var_max, ctx->d_err,
                                                s));
             *out = idx;
@@ -1924,7 +2042,7 @@ extern "C" int tkf_build_hit_index_noalloc(const tkf_config *cfg, const tkf_hits
     float4 *hxyzi = (float4 *)out->hit_xyzi;
     float2 *hvar = (float2 *)out->hit_var;
     if (segment_index(hits->n, n_segs, NB))
-        return launch_segment_index(g, *hits, n_sm, counts, out->event_off, hxyzi, hvar, (uint4 *)out->bin_sub,
+        return launch_segment_index(g, *hits, n_sm, counts, keys, out->event_off, hxyzi, hvar, (uint4 *)out->bin_sub,
                                     out->pos_of_hit, out->bin_off, (float2 *)out->var_max, err, s) == cudaSuccess
                    ? TKF_OK
                    : TKF_ERR_CUDA;

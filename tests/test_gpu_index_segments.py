@@ -115,6 +115,21 @@ def test_layers_whose_hits_are_not_in_order(n, order):
     _check(*_hits(rng, layer), layer, off)
 
 
+def test_events_with_their_layers_mixed_among_events_in_order():
+    """Every order within one batch, at sizes around the words and warps the layers are counted in, and a
+    segment of more than the large class holds."""
+    rng = np.random.default_rng(11)
+    layer = []
+    for k, n in enumerate([0, 1, 3, 4, 5, 31, 32, 33, 127, 129, 1023, 1024, 1025, 4099, 33000, 3 * L]):
+        for order in range(3):
+            a = np.sort(rng.integers(0, L, n))
+            layer.append(a if order == 0 else rng.permutation(a) if order == 1 else np.roll(np.arange(n) % L, k))
+    layer.append(rng.permutation(np.concatenate([np.full(38000, 7), np.arange(500) % L])))
+    off = np.concatenate([[0], np.cumsum([len(a) for a in layer])]).astype(np.int32)
+    layer = np.concatenate(layer)
+    _check(*_hits(rng, layer), layer, off)
+
+
 def test_a_dense_bin_and_many_equal_sixteenths():
     rng = np.random.default_rng(3)
     layer = np.repeat(np.arange(L), 3000)
