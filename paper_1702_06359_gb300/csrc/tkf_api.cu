@@ -459,6 +459,29 @@ k_bin_sort(const IndexGeom g, const int *bin_off, const int *ev_off, int n_bins_
 // of 160 k 120 / 102 us (ten blocks, each fetching 32 bytes for 4), 20 of 67 k 102 / 192 us, 160 of 55 k on
 // average 0.64 / 1.05 ms.  Passing over the hits of other layers instead: 41, 188, 506, 380 us, 2.25 ms.
 
+constexpr int kSegMaxBins = 4096;  // a bin's sixteenth in 16 bits
+constexpr int kSegThreads = 768, kSegThreadsBig = 1024;
+constexpr size_t kSegSmem = 112 * 1024, kSegSmemBig = 226 * 1024;  // two blocks per SM, one
+
+// Shared memory of a segment: a 16-bit counter for each sixteenth of each bin and one more (padded to
+// whole 16-byte words), and 4 bytes for each hit.
+__host__ __device__ __forceinline__ int seg_words(int n_bins) { return (n_bins * kSubBins + 8) / 8; }
+int segment_cap(int n_bins, size_t smem) { return ((int)smem - 16 * seg_words(n_bins)) / 4; }
+
+// The same with 2 bytes for each hit (their number in 16 bits).
+__host__ __device__ __forceinline__ int whole_cap(int n_bins)
+{
+    const int n = ((int)kSegSmemBig - 16 * seg_words(n_bins)) / 2;
+    return n < 65535 ? n : 65535;
+}
+// A segment of more hits is taken in parts, each some of its bins: a counter for each bin of the segment,
+// the part's sixteenths, 8 bytes for each of the part's hits.
+__host__ __device__ __forceinline__ int part_bin_words(int n_bins) { return (n_bins + 4) / 4; }
+__host__ __device__ __forceinline__ int part_cap(int n_bins)
+{
+    return ((int)kSegSmemBig - 16 * (part_bin_words(n_bins) + seg_words(n_bins))) / 8;
+}
+
 // The layers of hits i .. i + 3 (-1 outside h0 .. h1 - 1), as one word where the array is aligned to it.
 __device__ __forceinline__ int4 layer_word(const tkf_hits &h, bool aligned, int i, int h0, int h1)
 {
@@ -529,7 +552,7 @@ __global__ void __launch_bounds__(kLayerThreads) k_index_layers(const IndexGeom 
                     continue;
                 }
                 if (c != l[v][u - 1] || i == h0) {  // a run's length is its end minus its start
-                    atomicAdd(&s_runs[c], 1);
+                    if (atomicAdd(&s_runs[c], 1) > 0) s_mixed = 1;
                     atomicAdd(&s_cnt[c], -i);
                     s_start[c] = i;
                 }
@@ -538,9 +561,7 @@ __global__ void __launch_bounds__(kLayerThreads) k_index_layers(const IndexGeom 
         }
     }
     __syncthreads();
-    bool mixed = s_mixed;
-    for (int l = 0; l < g.L; ++l) mixed |= s_runs[l] > 1;
-    if (mixed) {  // block-uniform: count hit by hit, a thread's in bytes
+    if (s_mixed) {  // block-uniform: count hit by hit, a thread's in bytes
         static_assert(TKF_MAX_LAYERS == 16, "a byte of c for each layer");
         __syncthreads();
         if (tid < g.L) {
@@ -591,15 +612,6 @@ __global__ void __launch_bounds__(kLayerThreads) k_index_layers(const IndexGeom 
         seg_start[e * g.L + tid] = s_start[tid];
     }
 }
-
-constexpr int kSegMaxBins = 4096;  // a bin's sixteenth in 16 bits
-constexpr int kSegThreads = 768, kSegThreadsBig = 1024;
-constexpr size_t kSegSmem = 112 * 1024, kSegSmemBig = 226 * 1024;  // two blocks per SM, one
-
-// Shared memory of a segment: a 16-bit counter for each sixteenth of each bin and one more (padded to
-// whole 16-byte words), and 4 bytes for each hit.
-__host__ __device__ __forceinline__ int seg_words(int n_bins) { return (n_bins * kSubBins + 8) / 8; }
-int segment_cap(int n_bins, size_t smem) { return ((int)smem - 16 * seg_words(n_bins)) / 4; }
 
 __device__ __forceinline__ unsigned half16(const unsigned *w, unsigned k) { return (w[k >> 1] >> (16 * (k & 1))) & 0xFFFFu; }
 
@@ -665,9 +677,318 @@ template <int T, class A, class F> __device__ __forceinline__ void for_hits(cons
     }
 }
 
+// Turns the counts of a block's cells (two a 32-bit half, nw 16-byte words) into their ends: inclusive
+// scan; thread t owns a contiguous chunk of words, an odd number of them (a multiple of 8 would put every
+// lane's words in the same banks).  s_part: a word per warp.
+template <int T> __device__ __forceinline__ void cell_ends(uint4 *s_words, int nw, int *s_part)
+{
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int per = ((nw + T - 1) / T) | 1, c0 = min(tid * per, nw), c1 = min(c0 + per, nw);
+    unsigned sum = 0;  // both halves at once: no carry, the cells hold fewer than 2^16 hits
+    for (int k = c0; k < c1; ++k) {
+        const uint4 q = s_words[k];
+        sum += q.x + q.y + q.z + q.w;
+    }
+    const int mine = (int)((sum & 0xFFFFu) + (sum >> 16));
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_part[w] = incl;
+    __syncthreads();
+    unsigned run = (unsigned)(incl - mine);
+    for (int k = 0; k < w; ++k) run += (unsigned)s_part[k];
+    auto ends = [&](unsigned c) {  // both cells' ends from their counts
+        const unsigned a = run + (c & 0xFFFFu);
+        run = a + (c >> 16);
+        return a | (run << 16);
+    };
+    for (int k = c0; k < c1; ++k) {
+        uint4 q = s_words[k];
+        q.x = ends(q.x);
+        q.y = ends(q.y);
+        q.z = ends(q.z);
+        q.w = ends(q.w);
+        s_words[k] = q;
+    }
+    __syncthreads();
+}
+
+// The bin_sub word of bin b from the cells' starts (a bin's sixteenths are 8 words): the starts relative
+// to the bin's, a, as bytes.
+__device__ __forceinline__ uint4 bin_table(const uint4 *s_words, int b, unsigned &a)
+{
+    const uint4 q0 = s_words[2 * b], q1 = s_words[2 * b + 1];
+    a = q0.x & 0xFFFFu;
+    const unsigned n = half16((const unsigned *)s_words, (b + 1) * kSubBins) - a;
+    const unsigned aa = a | (a << 16);  // no borrow: starts do not decrease
+    auto bytes = [](unsigned u, unsigned v, unsigned x) {  // halves u.hi, v.lo, v.hi, x.lo
+        return __byte_perm(__byte_perm(u, v, 0x0642), x, 0x4210);
+    };
+    const unsigned d0 = q0.x - aa, d1 = q0.y - aa, d2 = q0.z - aa, d3 = q0.w - aa;
+    const unsigned d4 = q1.x - aa, d5 = q1.y - aa, d6 = q1.z - aa, d7 = q1.w - aa;
+    const uint4 sub = make_uint4(bytes(d0, d1, d2), bytes(d2, d3, d4), bytes(d4, d5, d6), bytes(d6, d7, 0u));
+    return n > 255u ? make_uint4(~0u, ~0u, ~0u, ~0u) : sub;
+}
+
+// The block's largest variances (the order of non-negative floats is that of their bits); s_mu, s_mv: zero.
+__device__ __forceinline__ int2 block_max(float mu, float mv, int *s_mu, int *s_mv)
+{
+    const unsigned ru = __reduce_max_sync(0xffffffffu, __float_as_uint(mu)),
+                   rv = __reduce_max_sync(0xffffffffu, __float_as_uint(mv));
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(s_mu, (int)ru);
+        atomicMax(s_mv, (int)rv);
+    }
+    __syncthreads();
+    return make_int2(*s_mu, *s_mv);
+}
+
+// The arrays of a segment index.
+struct SegIndex {
+    const int *count, *start;  // per segment
+    int *list;
+    float4 *hxyzi;
+    float2 *hvar;
+    uint4 *bin_sub;
+    int *pos_of_hit, *bin_off;
+    float2 *var_max;
+};
+
+// Hits whose layer is out of range have no bin, and the event's segments start at its first position, so
+// as many positions stay free behind its last segment, inside the range of its last bin.  They take
+// hits that no window holds (its tests are comparisons, which fail on NaN).
+template <int T> __device__ __forceinline__ void fill_free(const SegIndex &x, int pos, int end)
+{
+    for (pos += threadIdx.x; pos < end; pos += T) {
+        x.hxyzi[pos] = make_float4(CUDART_NAN_F, CUDART_NAN_F, CUDART_NAN_F, __int_as_float(0));
+        x.hvar[pos] = make_float2(0.f, 0.f);
+    }
+}
+
+// A segment too large for the keys of its hits in shared memory, by one block: they wait in pos_of_hit.
+// Up to 65535 hits it is ordered at once, as a smaller one.  Of a larger one the hits per bin are counted
+// first; then its bins are taken in parts, whose hits are collected and ordered.  A bin that is too large by
+// itself is ordered by words in global memory.  What bounds it: one block's scattered accesses, 32
+// bytes for 4.  A layer of 40 k / 110 k hits beside nine of 4 k: 126 / 689 us, ten layers of 67 k / 270 k 0.39 /
+// 3.6 ms; by the multi-launch kernels 166 / 574 us and 0.34 / 75.6 ms, with all hits ordered by words 1183 /
+// 9193 us and 3.5 / 57 ms.  Measured and not taken: parts for other blocks, each binning the whole segment (109 /
+// 227 us, 0.20 / 1.6 ms), because the blocks that look for parts made every batch slower (20 events
+// 44.2 -> 46.8 us, 512 events 720 -> 728); hits placed into their bins and ordered there in place 0.82 ms for
+// the layer of 110 k.
+template <int T>
+__device__ __noinline__ void segment_large(const IndexGeom &g, const tkf_hits &h, const SegIndex &x, int seg, int cnt,
+                                           int base, uint4 *s_words, int *s_part, int *s_mu, int *s_mv)
+{
+    __shared__ int s_n;
+    const unsigned full = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nb = g.n_bins;
+    const int e = seg / g.L, l = seg - e * g.L, h0 = h.event_off[e];
+    const int start = x.start[seg], *ids = x.list + base;
+    auto at = [=](int j) { return start < 0 ? ids[j] : start + j; };
+    const float rl = g.radius[l];
+    const bool disk = (g.disk_mask >> l) & 1u;
+    const size_t b0 = (size_t)seg * nb;
+    const int cap = part_cap(nb);
+    int *s_bin = (int *)s_words;  // [nb + 1]
+    uint4 *s_cells = s_words + part_bin_words(nb);
+    unsigned *s_cell = (unsigned *)s_cells;
+    int *s_id = (int *)(s_cells + seg_words(nb));
+    unsigned short *s_key = (unsigned short *)(s_id + cap), *s_ord = s_key + cap;
+    float mu = 0.f, mv = 0.f;
+    auto done = [&]() {
+        const int2 most = block_max(mu, mv, s_mu, s_mv);
+        if (tid == 0) x.var_max[seg] = make_float2(__int_as_float(most.x), __int_as_float(most.y));
+    };
+    if (cnt <= whole_cap(nb)) {
+        const int nw = seg_words(nb);
+        unsigned *s_all = (unsigned *)s_words;
+        unsigned short *s_place = (unsigned short *)(s_words + nw);
+        for (int k = tid; k < nw; k += T) s_words[k] = make_uint4(0u, 0u, 0u, 0u);
+        if (tid == 0) *s_mu = *s_mv = 0;
+        __syncthreads();
+        for_hits<T>(h, at, cnt, [&](int j, float hx, float hy, float hz) {
+            const unsigned key = hit_key(g, rl, disk, hx, hy, hz);
+            x.pos_of_hit[at(j)] = (int)key;
+            atomicAdd(&s_all[key >> 1], key & 1 ? 0x10000u : 1u);
+        });
+        __syncthreads();
+        cell_ends<T>(s_words, nw, s_part);
+        for (int j = tid; j < cnt; j += T) {
+            const unsigned key = (unsigned)x.pos_of_hit[at(j)], sh = 16 * (key & 1);
+            const unsigned old = atomicSub(&s_all[key >> 1], 1u << sh);
+            s_place[((old >> sh) & 0xFFFFu) - 1] = (unsigned short)j;
+        }
+        __syncthreads();
+        for (int b = tid; b < nb; b += T) {
+            unsigned rel;
+            x.bin_sub[b0 + b] = bin_table(s_words, b, rel);
+            x.bin_off[b0 + b] = base + (int)rel;
+        }
+        for_hits<T>(h, at, cnt, [&](int j, float hx, float hy, float hz) {
+            const int i = at(j);
+            const unsigned key = (unsigned)x.pos_of_hit[i];
+            const float vu = h.var_u[i], vv = h.var_v[i];
+            const int a0 = (int)half16(s_all, key), a1 = (int)half16(s_all, key + 1);
+            int pos = base + a0;
+            if (a1 - a0 > 1)
+                for (int t = a0; t < a1; ++t) pos += s_place[t] < j;
+            x.hxyzi[pos] = make_float4(hx, hy, hz, __int_as_float(i - h0));
+            x.hvar[pos] = make_float2(vu, vv);
+            x.pos_of_hit[i] = pos;
+            mu = fmaxf(mu, vu);
+            mv = fmaxf(mv, vv);
+        });
+        done();
+        return;
+    }
+    constexpr int kWaiting = (int)0x80000000u;  // with a key in pos_of_hit: not placed yet
+    for (int b = tid; b <= nb; b += T) s_bin[b] = 0;
+    if (tid == 0) *s_mu = *s_mv = 0;
+    __syncthreads();
+    // (1) hits per bin, and where the bins start
+    for_hits<T>(h, at, cnt, [&](int j, float hx, float hy, float hz) {
+        const unsigned key = hit_key(g, rl, disk, hx, hy, hz);
+        x.pos_of_hit[at(j)] = (int)key | kWaiting;
+        atomicAdd(&s_bin[key / kSubBins], 1);
+    });
+    __syncthreads();
+    const int per = (nb + T) / T, c0 = min(tid * per, nb + 1), c1 = min(c0 + per, nb + 1);
+    int sum = 0;
+    for (int b = c0; b < c1; ++b) sum += s_bin[b];
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(full, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_part[w] = incl;
+    __syncthreads();
+    int run = incl - sum;
+    for (int k = 0; k < w; ++k) run += s_part[k];
+    for (int b = c0; b < c1; ++b) {
+        const int c = s_bin[b];
+        s_bin[b] = run;
+        run += c;
+    }
+    __syncthreads();
+    for (int first = 0, end; first < nb; first = end) {
+        // the part: bins first .. end - 1, and their hits, own of them from position a of the segment on
+        const int a = s_bin[first];
+        end = first + 1;
+        for (int hi = nb; end < hi;) {  // the most bins whose hits fit, or one
+            const int mid = (end + hi + 1) >> 1;
+            if (s_bin[mid] - a <= cap) end = mid; else hi = mid - 1;
+        }
+        const int own = s_bin[end] - a;
+        // f(hit's place in the segment, hit, key, its number) for the part's hits, numbered from s_n on
+        auto each_own = [&](auto f) {
+            constexpr int U = 4;
+            for (int q0 = 0; q0 < cnt; q0 += U * T) {  // every thread takes every turn
+                int i[U], key[U], total = 0;
+                unsigned in[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    i[u] = at(min(q0 + u * T + tid, cnt - 1));
+                    key[u] = x.pos_of_hit[i[u]];
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const unsigned k = (unsigned)(key[u] & ~kWaiting);
+                    in[u] = __ballot_sync(full, q0 + u * T + tid < cnt && key[u] < 0 && k >= (unsigned)first * kSubBins &&
+                                                    k < (unsigned)end * kSubBins);
+                    total += __popc(in[u]);
+                }
+                int m = 0;  // (one number a hit taken from s_n: 17 k of them in turn)
+                if (lane == 0 && total > 0) m = atomicAdd(&s_n, total);
+                m = __shfl_sync(full, m, 0);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (in[u] >> lane & 1u)
+                        f(q0 + u * T + tid, i[u], (unsigned)(key[u] & ~kWaiting), m + __popc(in[u] & ((1u << lane) - 1u)));
+                    m += __popc(in[u]);
+                }
+            }
+        };
+        if (tid == 0) s_n = 0;
+        if (own <= cap) {
+            const int nw = seg_words(end - first);
+            for (int k = tid; k < nw; k += T) s_cells[k] = make_uint4(0u, 0u, 0u, 0u);
+            __syncthreads();
+            // (2) the part's hits, in no order: place in the segment and sixteenth
+            each_own([&](int j, int, unsigned key, int m) {
+                key -= first * kSubBins;
+                s_id[m] = j;
+                s_key[m] = (unsigned short)key;
+                atomicAdd(&s_cell[key >> 1], key & 1 ? 0x10000u : 1u);
+            });
+            __syncthreads();
+            cell_ends<T>(s_cells, nw, s_part);
+            for (int m = tid; m < own; m += T) {
+                const unsigned key = s_key[m], sh = 16 * (key & 1);
+                const unsigned old = atomicSub(&s_cell[key >> 1], 1u << sh);
+                s_ord[((old >> sh) & 0xFFFFu) - 1] = (unsigned short)m;
+            }
+            __syncthreads();
+            for (int b = first + tid; b < end; b += T) {
+                unsigned rel;
+                x.bin_sub[b0 + b] = bin_table(s_cells, b - first, rel);
+                x.bin_off[b0 + b] = base + a + (int)rel;
+            }
+            // (3) to their places: a sixteenth's hits in the order of their ids
+            for_hits<T>(h, [&](int m) { return at(s_id[m]); }, own, [&](int m, float hx, float hy, float hz) {
+                const unsigned key = s_key[m];
+                const int a0 = (int)half16(s_cell, key), a1 = (int)half16(s_cell, key + 1), j = s_id[m];
+                int pos = base + a + a0;
+                if (a1 - a0 > 1)
+                    for (int t = a0; t < a1; ++t) pos += s_id[s_ord[t]] < j;
+                const int i = at(j);
+                const float vu = h.var_u[i], vv = h.var_v[i];
+                x.hxyzi[pos] = make_float4(hx, hy, hz, __int_as_float(i - h0));
+                x.hvar[pos] = make_float2(vu, vv);
+                x.pos_of_hit[i] = pos;
+                mu = fmaxf(mu, vu);
+                mv = fmaxf(mv, vv);
+            });
+        } else {  // one bin: words of sixteenth and id in its part of hvar
+            // (the id whole: an event over the hit limit, which is reported, has ids beyond 23 bits, and two
+            // words that compared equal would leave a position of the index unwritten)
+            unsigned long long *g_ord = (unsigned long long *)(x.hvar + base + a);
+            auto order_word = [&](unsigned key, int i) {
+                return ((unsigned long long)(key & (kSubBins - 1)) << 32) | (unsigned)(i - h0);
+            };
+            __syncthreads();
+            each_own([&](int, int i, unsigned key, int m) { g_ord[m] = order_word(key, i); });
+            __syncthreads();
+            if (tid == 0) {
+                x.bin_off[b0 + first] = base + a;
+                x.bin_sub[b0 + first] = make_uint4(~0u, ~0u, ~0u, ~0u);  // more than 255 hits
+            }
+            each_own([&](int, int i, unsigned key, int) {
+                const unsigned long long word = order_word(key, i);
+                int pos = base + a;
+                for (int t = 0; t < own; ++t) pos += g_ord[t] < word;
+                x.pos_of_hit[i] = pos;
+                const float vu = h.var_u[i], vv = h.var_v[i];
+                x.hxyzi[pos] = make_float4(h.x[i], h.y[i], h.z[i], __int_as_float(i - h0));
+                mu = fmaxf(mu, vu);
+                mv = fmaxf(mv, vv);
+            });
+            __syncthreads();  // every word has been compared: hvar takes the variances
+            for (int m = tid; m < own; m += T) {
+                const int i = h0 + __float_as_int(x.hxyzi[base + a + m].w);
+                x.hvar[base + a + m] = make_float2(h.var_u[i], h.var_v[i]);
+            }
+        }
+        __syncthreads();  // the shared memory is the next part's
+    }
+    done();
+}
+
 // The segment of one (event, layer).  A launch takes the segments with lo < hits <= cap, held in shared
-// memory; the last launch (kLast) also the larger ones: only their bins are counted there, the
-// hits' keys live in pos_of_hit and their order words in hvar until the final positions are known.
+// memory; the last launch (kLast) also the larger ones (segment_large).
 //
 // What bounds it: the latency of its phases (loads, counting, scan, tables, placing, each behind a
 // barrier) with 73 % of the warps resident and 40 % issue; 512 events (23.5 M hits) move 1.7 GB in 0.70
@@ -679,206 +1000,88 @@ template <int T, class A, class F> __device__ __forceinline__ void for_hits(cons
 // 0.73 ms.
 template <int T, int kPerSM, bool kLast>
 __global__ void __launch_bounds__(T, kPerSM)
-k_index_segment(const __grid_constant__ IndexGeom g, const tkf_hits h, const int *seg_count,
-                const int *seg_start, int *list, int lo, int cap, float4 *hxyzi, float2 *hvar, uint4 *bin_sub, int *pos_of_hit, int *bin_off, float2 *var_max)
+k_index_segment(const __grid_constant__ IndexGeom g, const __grid_constant__ tkf_hits h,
+                const __grid_constant__ SegIndex x, int lo, int cap)
 {
     extern __shared__ uint4 s_words[];
     __shared__ int s_part[T / 32], s_mu, s_mv;
     after_previous();
-    const unsigned full = 0xffffffffu;
-    const int seg = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int cnt = seg_count[seg];
-    const bool fast = cnt <= cap && cnt < 65536;
-    if (fast ? cnt <= lo : !kLast) return;
+    const int seg = blockIdx.x, tid = threadIdx.x;
+    const int cnt = x.count[seg];
+    if (cnt <= lo || (!kLast && cnt > cap)) return;
     const int e = seg / g.L, l = seg - e * g.L;
-    const int h0 = h.event_off[e];
+    const int h0 = h.event_off[e], h1 = h.event_off[e + 1];
     int base = h0;
-    for (int k = 0; k < l; ++k) base += seg_count[e * g.L + k];
-    const int start = seg_start[seg];
-    if (start < 0) list_layer<T>(h, l, h0, h.event_off[e + 1], list + base, s_part);
+    for (int k = 0; k < l; ++k) base += x.count[e * g.L + k];
+    const int start = x.start[seg], *ids = x.list + base;
+    if (seg == g.n_events * g.L - 1 && tid == 0) x.bin_off[(size_t)(seg + 1) * g.n_bins] = base + cnt;
+    if (l == g.L - 1) fill_free<T>(x, base + cnt, h1);
+    if (kLast && cnt > cap) {
+        if (start < 0) list_layer<T>(h, l, h0, h1, x.list + base, s_part);
+        segment_large<T>(g, h, x, seg, cnt, base, s_words, s_part, &s_mu, &s_mv);
+        return;
+    }
     // the segment's hits in the order of their ids: consecutive, or listed
     auto each_way = [&](auto f) {
-        if (start < 0)
-            f([=](int j) { return list[base + j]; });
-        else
+        if (__builtin_expect(start >= 0, 1))
             f([=](int j) { return start + j; });
+        else
+            f([=](int j) { return ids[j]; });
     };
     const float rl = g.radius[l];
     const bool disk = (g.disk_mask >> l) & 1u;
     const size_t b0 = (size_t)seg * g.n_bins;
     if (tid == 0) s_mu = s_mv = 0;
-    if (seg == g.n_events * g.L - 1 && tid == 0) bin_off[b0 + g.n_bins] = base + cnt;
     float mu = 0.f, mv = 0.f;
-    if (fast) {
-        const int nw = seg_words(g.n_bins);
-        unsigned *s_cell = (unsigned *)s_words;  // two cells a word
-        unsigned short *s_key = (unsigned short *)(s_words + nw), *s_ord = s_key + cap;
-        for (int k = tid; k < nw; k += T) s_words[k] = make_uint4(0u, 0u, 0u, 0u);
-        __syncthreads();
-        // (1) the sixteenth of every hit; hits per sixteenth
-        each_way([&](auto at) {
-            for_hits<T>(h, at, cnt, [&](int j, float x, float y, float z) {
-                const unsigned key = hit_key(g, rl, disk, x, y, z);
-                s_key[j] = (unsigned short)key;
-                atomicAdd(&s_cell[key >> 1], key & 1 ? 0x10000u : 1u);
-            });
+    const int nw = seg_words(g.n_bins);
+    unsigned *s_cell = (unsigned *)s_words;  // two cells a word
+    unsigned short *s_key = (unsigned short *)(s_words + nw), *s_ord = s_key + cap;
+    for (int k = tid; k < nw; k += T) s_words[k] = make_uint4(0u, 0u, 0u, 0u);
+    if (__builtin_expect(start < 0, 0)) list_layer<T>(h, l, h0, h1, x.list + base, s_part);
+    __syncthreads();
+    // (1) the sixteenth of every hit; hits per sixteenth
+    each_way([&](auto at) {
+        for_hits<T>(h, at, cnt, [&](int j, float hx, float hy, float hz) {
+            const unsigned key = hit_key(g, rl, disk, hx, hy, hz);
+            s_key[j] = (unsigned short)key;
+            atomicAdd(&s_cell[key >> 1], key & 1 ? 0x10000u : 1u);
         });
-        __syncthreads();
-        // (2) inclusive scan: the end of every sixteenth; thread t owns a contiguous chunk of words, an
-        // odd number of them (a multiple of 8 would put every lane's words in the same banks)
-        const int per = ((nw + T - 1) / T) | 1, c0 = min(tid * per, nw), c1 = min(c0 + per, nw);
-        unsigned sum = 0;  // both halves at once: no carry, the segment has fewer than 2^16 hits
-        for (int k = c0; k < c1; ++k) {
-            const uint4 q = s_words[k];
-            sum += q.x + q.y + q.z + q.w;
-        }
-        const int mine = (int)((sum & 0xFFFFu) + (sum >> 16));
-        int incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(full, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane == 31) s_part[w] = incl;
-        __syncthreads();
-        unsigned run = (unsigned)(incl - mine);
-        for (int k = 0; k < w; ++k) run += (unsigned)s_part[k];
-        auto ends = [&](unsigned c) {  // both cells' ends from their counts
-            const unsigned a = run + (c & 0xFFFFu);
-            run = a + (c >> 16);
-            return a | (run << 16);
-        };
-        for (int k = c0; k < c1; ++k) {
-            uint4 q = s_words[k];
-            q.x = ends(q.x);
-            q.y = ends(q.y);
-            q.z = ends(q.z);
-            q.w = ends(q.w);
-            s_words[k] = q;
-        }
-        __syncthreads();
-        // (3) hits into their sixteenths, from the end down: the cells then hold the starts
-        for (int j = tid; j < cnt; j += T) {
-            const unsigned key = s_key[j], sh = 16 * (key & 1);
-            const unsigned old = atomicSub(&s_cell[key >> 1], 1u << sh);
-            s_ord[((old >> sh) & 0xFFFFu) - 1] = (unsigned short)j;
-        }
-        __syncthreads();
-        // (4) the bin tables: a bin's sixteenths are 8 words; their starts relative to the bin's, as bytes
-        for (int b = tid; b < g.n_bins; b += T) {
-            const uint4 q0 = s_words[2 * b], q1 = s_words[2 * b + 1];
-            const unsigned a = q0.x & 0xFFFFu, n = half16(s_cell, (b + 1) * kSubBins) - a;
-            bin_off[b0 + b] = base + (int)a;
-            const unsigned aa = a | (a << 16);  // no borrow: starts do not decrease
-            auto bytes = [](unsigned u, unsigned v, unsigned x) {  // halves u.hi, v.lo, v.hi, x.lo
-                return __byte_perm(__byte_perm(u, v, 0x0642), x, 0x4210);
-            };
-            const unsigned d0 = q0.x - aa, d1 = q0.y - aa, d2 = q0.z - aa, d3 = q0.w - aa;
-            const unsigned d4 = q1.x - aa, d5 = q1.y - aa, d6 = q1.z - aa, d7 = q1.w - aa;
-            uint4 sub = make_uint4(bytes(d0, d1, d2), bytes(d2, d3, d4), bytes(d4, d5, d6), bytes(d6, d7, 0u));
-            if (n > 255u) sub = make_uint4(~0u, ~0u, ~0u, ~0u);
-            bin_sub[b0 + b] = sub;
-        }
-        // (5) the hits to their places: a sixteenth's hits in the order of their ids
-        each_way([&](auto at) {
-            for_hits<T>(h, at, cnt, [&](int j, float x, float y, float z) {
-                const unsigned key = s_key[j];
-                const int a0 = (int)half16(s_cell, key), a1 = (int)half16(s_cell, key + 1);
-                int pos = base + a0;
-                if (a1 - a0 > 1)
-                    for (int t = a0; t < a1; ++t) pos += s_ord[t] < j;
-                const int i = at(j);
-                const float vu = h.var_u[i], vv = h.var_v[i];
-                hxyzi[pos] = make_float4(x, y, z, __int_as_float(i - h0));
-                hvar[pos] = make_float2(vu, vv);
-                pos_of_hit[i] = pos;
-                mu = fmaxf(mu, vu);
-                mv = fmaxf(mv, vv);
-            });
-        });
-    } else {
-        int *s_bin = (int *)s_words;  // counts, then cursors: start of a bin, then its end
-        // order word q: sixteenth and id, the id whole (an event over the hit limit, which is reported, has ids
-        // beyond 23 bits; two words that compared equal would leave a position of the index unwritten)
-        unsigned long long *g_ord = (unsigned long long *)(hvar + base);
-        auto order_word = [&](unsigned key, int i) {
-            return ((unsigned long long)(key & (kSubBins - 1)) << 32) | (unsigned)(i - h0);
-        };
-        for (int b = tid; b < g.n_bins; b += T) s_bin[b] = 0;
-        __syncthreads();
-        for (int j = tid; j < cnt; j += T) {
-            const int i = start < 0 ? list[base + j] : start + j;
-            const unsigned key = hit_key(g, rl, disk, h.x[i], h.y[i], h.z[i]);
-            pos_of_hit[i] = (int)key;
-            atomicAdd(&s_bin[key / kSubBins], 1);
-        }
-        __syncthreads();
-        const int per = (g.n_bins + T - 1) / T, c0 = min(tid * per, g.n_bins), c1 = min(c0 + per, g.n_bins);
-        int sum = 0;
-        for (int b = c0; b < c1; ++b) sum += s_bin[b];
-        int incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(full, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane == 31) s_part[w] = incl;
-        __syncthreads();
-        int run = incl - sum;
-        for (int k = 0; k < w; ++k) run += s_part[k];
-        for (int b = c0; b < c1; ++b) {
-            const int c = s_bin[b];
-            s_bin[b] = run;
-            run += c;
-        }
-        __syncthreads();
-        for (int j = tid; j < cnt; j += T) {
-            const int i = start < 0 ? list[base + j] : start + j;
-            const unsigned key = (unsigned)pos_of_hit[i];
-            g_ord[atomicAdd(&s_bin[key / kSubBins], 1)] = order_word(key, i);
-        }
-        __syncthreads();
-        for (int b = tid; b < g.n_bins; b += T) {
-            const int a0 = b ? s_bin[b - 1] : 0, a1 = s_bin[b];
-            bin_off[b0 + b] = base + a0;
-            bin_sub[b0 + b] = sub_starts([&](int t) { return (int)(g_ord[t] >> 32) << 23; }, a0, a1);
-        }
-        for (int j = tid; j < cnt; j += T) {
-            const int i = start < 0 ? list[base + j] : start + j;
-            const unsigned key = (unsigned)pos_of_hit[i], b = key / kSubBins;
-            const unsigned long long word = order_word(key, i);
-            const int a0 = b ? s_bin[b - 1] : 0, a1 = s_bin[b];
-            int pos = base + a0;
-            for (int t = a0; t < a1; ++t) pos += g_ord[t] < word;
-            pos_of_hit[i] = pos;
-        }
-        __syncthreads();  // every word has been compared: hvar takes the variances
-        for (int j = tid; j < cnt; j += T) {
-            const int i = start < 0 ? list[base + j] : start + j;
-            const int pos = pos_of_hit[i];
-            const float vu = h.var_u[i], vv = h.var_v[i];
-            hxyzi[pos] = make_float4(h.x[i], h.y[i], h.z[i], __int_as_float(i - h0));
-            hvar[pos] = make_float2(vu, vv);
-            mu = fmaxf(mu, vu);
-            mv = fmaxf(mv, vv);
-        }
-    }
-    // Hits whose layer is out of range have no bin, and the event's segments start at its first position, so
-    // as many positions stay free behind its last segment, inside the range of its last bin.  They take
-    // hits that no window holds (its tests are comparisons, which fail on NaN).
-    if (l == g.L - 1)
-        for (int pos = base + cnt + tid, end = h.event_off[e + 1]; pos < end; pos += T) {
-            hxyzi[pos] = make_float4(CUDART_NAN_F, CUDART_NAN_F, CUDART_NAN_F, __int_as_float(0));
-            hvar[pos] = make_float2(0.f, 0.f);
-        }
-    // the largest variances (the order of non-negative floats is that of their bits)
-    const unsigned ru = __reduce_max_sync(full, __float_as_uint(mu)), rv = __reduce_max_sync(full, __float_as_uint(mv));
-    if (lane == 0) {
-        atomicMax(&s_mu, (int)ru);
-        atomicMax(&s_mv, (int)rv);
+    });
+    __syncthreads();
+    // (2) the end of every sixteenth
+    cell_ends<T>(s_words, nw, s_part);
+    // (3) hits into their sixteenths, from the end down: the cells then hold the starts
+    for (int j = tid; j < cnt; j += T) {
+        const unsigned key = s_key[j], sh = 16 * (key & 1);
+        const unsigned old = atomicSub(&s_cell[key >> 1], 1u << sh);
+        s_ord[((old >> sh) & 0xFFFFu) - 1] = (unsigned short)j;
     }
     __syncthreads();
-    if (tid == 0) var_max[seg] = make_float2(__int_as_float(s_mu), __int_as_float(s_mv));
+    // (4) the bin tables: a bin's sixteenths are 8 words; their starts relative to the bin's, as bytes
+    for (int b = tid; b < g.n_bins; b += T) {
+        unsigned a;
+        x.bin_sub[b0 + b] = bin_table(s_words, b, a);
+        x.bin_off[b0 + b] = base + (int)a;
+    }
+    // (5) the hits to their places: a sixteenth's hits in the order of their ids
+    each_way([&](auto at) {
+        for_hits<T>(h, at, cnt, [&](int j, float hx, float hy, float hz) {
+            const unsigned key = s_key[j];
+            const int a0 = (int)half16(s_cell, key), a1 = (int)half16(s_cell, key + 1);
+            int pos = base + a0;
+            if (a1 - a0 > 1)
+                for (int t = a0; t < a1; ++t) pos += s_ord[t] < j;
+            const int i = at(j);
+            const float vu = h.var_u[i], vv = h.var_v[i];
+            x.hxyzi[pos] = make_float4(hx, hy, hz, __int_as_float(i - h0));
+            x.hvar[pos] = make_float2(vu, vv);
+            x.pos_of_hit[i] = pos;
+            mu = fmaxf(mu, vu);
+            mv = fmaxf(mv, vv);
+        });
+    });
+    const int2 most = block_max(mu, mv, &s_mu, &s_mv);
+    if (tid == 0) x.var_max[seg] = make_float2(__int_as_float(most.x), __int_as_float(most.y));
 }
 
 // Whether a batch is indexed by k_index_segment: its sixteenths fit 16 bits and its segments, on
@@ -890,20 +1093,19 @@ bool segment_index(int n_hits, size_t n_segs, int n_bins)
     return n_bins <= kSegMaxBins && n_bins >= 4 && (size_t)n_hits <= n_segs * 16384;
 }
 
-// seg: 2 n_segs words of scratch; list: one word for each hit.
-cudaError_t launch_segment_index(const IndexGeom &g, const tkf_hits &h, int sm_count, int *seg, int *list, int *ev_off,
-                                 float4 *hxyzi, float2 *hvar, uint4 *bin_sub, int *pos_of_hit, int *bin_off,
-                                 float2 *var_max, int *err, cudaStream_t s)
+// scratch: 2 n_segs words; x.list: a word for each hit.
+cudaError_t launch_segment_index(const IndexGeom &g, const tkf_hits &h, int sm_count, int *scratch, SegIndex x, int *ev_off,
+                                 int *err, cudaStream_t s)
 {
     const unsigned n_segs = (unsigned)(g.n_events * g.L);
-    int *cnt = seg, *start = seg + n_segs;
-    cudaError_t e = launch_next(k_index_layers, (unsigned)g.n_events, kLayerThreads, 0, s, g, h, ev_off, cnt, start, err);
+    int *count = scratch, *start = count + n_segs;
+    x.count = count;
+    x.start = start;
+    cudaError_t e = launch_next(k_index_layers, (unsigned)g.n_events, kLayerThreads, 0, s, g, h, ev_off, count, start, err);
     int lo = -1;
     auto take = [&](auto kern, int threads, size_t smem) {
         const int hi = segment_cap(g.n_bins, smem);
-        if (e == cudaSuccess)
-            e = launch_next(kern, n_segs, threads, smem, s, g, h, cnt, start, list, lo, hi, hxyzi, hvar, bin_sub,
-                            pos_of_hit, bin_off, var_max);
+        if (e == cudaSuccess) e = launch_next(kern, n_segs, threads, smem, s, g, h, x, lo, hi);
         lo = std::max(hi, -1);
     };
     if ((int)n_segs > sm_count) take(k_index_segment<kSegThreads, 2, false>, kSegThreads, kSegSmem);
@@ -1604,9 +1806,9 @@ int tkf_build_hit_index(tkf_ctx *ctx, const tkf_hits *hits, tkf_hit_index **out,
         cudaStream_t s = (cudaStream_t)stream;
         const IndexGeom g = index_geom(c, hits->n_events);
         if (segment_index(hits->n, n_segs, NB)) {
-            TKF_CUDA(ctx, launch_segment_index(g, *hits, ctx->sm_count, idx->counts, idx->keys, idx->ev_off, idx->hxyzi, idx->hvar,
-                                               idx->bin_sub, idx->pos_of_hit, idx->bin_off, idx->var_max, ctx->d_err,
-                                               s));
+            const SegIndex x{nullptr,      nullptr,         idx->keys,    idx->hxyzi,  idx->hvar,
+                             idx->bin_sub, idx->pos_of_hit, idx->bin_off, idx->var_max};
+            TKF_CUDA(ctx, launch_segment_index(g, *hits, ctx->sm_count, idx->counts, x, idx->ev_off, ctx->d_err, s));
             *out = idx;
             return TKF_OK;
         }
@@ -2041,11 +2243,11 @@ extern "C" int tkf_build_hit_index_noalloc(const tkf_config *cfg, const tkf_hits
     cudaStream_t s = (cudaStream_t)stream;
     float4 *hxyzi = (float4 *)out->hit_xyzi;
     float2 *hvar = (float2 *)out->hit_var;
-    if (segment_index(hits->n, n_segs, NB))
-        return launch_segment_index(g, *hits, n_sm, counts, keys, out->event_off, hxyzi, hvar, (uint4 *)out->bin_sub,
-                                    out->pos_of_hit, out->bin_off, (float2 *)out->var_max, err, s) == cudaSuccess
-                   ? TKF_OK
-                   : TKF_ERR_CUDA;
+    if (segment_index(hits->n, n_segs, NB)) {
+        const SegIndex x{nullptr, nullptr, keys, hxyzi, hvar, (uint4 *)out->bin_sub, out->pos_of_hit, out->bin_off,
+                         (float2 *)out->var_max};
+        return launch_segment_index(g, *hits, n_sm, counts, x, out->event_off, err, s) == cudaSuccess ? TKF_OK : TKF_ERR_CUDA;
+    }
     if (cudaMemcpyAsync(out->event_off, hits->event_off, (hits->n_events + 1) * sizeof(int), cudaMemcpyDeviceToDevice,
                         s) != cudaSuccess)
         return TKF_ERR_CUDA;
