@@ -108,9 +108,11 @@ int issue(tkf_pipeline *p, const tkf_hits *hits, const int32_t *seed_hits, const
     if (capturing && (cudaEventRecord(p->fork, s) != cudaSuccess || cudaStreamWaitEvent(p->side, p->fork, 0) != cudaSuccess))
         return fail(ctx, TKF_ERR_CUDA, "pipeline: fork");
     int st = tkf::seed_and_fit(ctx, hits, seed_hits, first - 1, &seeds, (tkf_stream)seed_stream);
-    if (st || (st = tkf_build_hit_index(ctx, hits, &p->idx, (tkf_stream)s))) return st;
-    if (capturing && (cudaEventRecord(p->join, p->side) != cudaSuccess || cudaStreamWaitEvent(s, p->join, 0) != cudaSuccess))
-        return fail(ctx, TKF_ERR_CUDA, "pipeline: join");
+    if (!st) st = tkf_build_hit_index(ctx, hits, &p->idx, (tkf_stream)s);
+    // (a refused step joins its branch as well: a capture that ends without leaves its error to the next call)
+    if (capturing && (cudaEventRecord(p->join, p->side) != cudaSuccess || cudaStreamWaitEvent(s, p->join, 0) != cudaSuccess) && !st)
+        st = fail(ctx, TKF_ERR_CUDA, "pipeline: join");
+    if (st) return st;
     // events around the building kernel (event-record nodes when captured into the graph)
     const unsigned flag = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (cudaEventRecordWithFlags(p->build_ev[0], s, flag) != cudaSuccess)

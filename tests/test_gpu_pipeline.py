@@ -248,3 +248,53 @@ def test_two_step_pipeline_equals_direct_calls():
     assert np.all(ids == b.trk_hits, axis=1).mean() >= 0.97
     pipe.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("wrong", [dict(x=None), dict(event_off=None), dict(n_events=0)], ids=lambda w: next(iter(w)))
+def test_a_refused_run_leaves_pipeline_and_context_usable(wrong):
+    """The hits are checked inside the step, behind the fork of the captured graph's branch: the refusal is
+    the call's own, and neither the next direct call nor the next run reports anything of it."""
+    import ctypes as C
+    b = _batch(63, n_events=3)
+    ctx = tkf.Context(tkf.default_config())
+    L, n = ctx.cfg.n_layers, b.n_tracks
+    dh = device_hits(b)
+    sh = torch.as_tensor(np.ascontiguousarray(b.trk_hits[:, :3].T), dtype=torch.int32, device="cuda")
+    se = torch.as_tensor(b.trk_event, dtype=torch.int32, device="cuda")
+    pipe = tkf.DevicePipeline(ctx, b.n_hits, b.n_events, n, use_graph=True)
+    hs = dh.struct()
+    for k, v in wrong.items():
+        setattr(hs, k, v)
+    for _ in range(2):
+        code = tkf.lib().tkf_pipeline_run(pipe.handle, C.byref(hs), C.c_void_p(sh.data_ptr()), C.c_void_p(se.data_ptr()), n, None)
+        assert code == tkf.ERR_INVALID
+        built, final = _direct(ctx, b, dh, sh, se)
+    pipe.run(dh, sh, se, n)
+    torch.cuda.synchronize()
+    bt, ft = _pipe_out(pipe, L, n)
+    assert torch.equal(bt["hit_idx"], built.hit_idx) and torch.equal(ft["par"], final.par) and torch.equal(ft["cov"], final.cov)
+
+
+def test_a_run_refused_by_the_index_leaves_no_error_behind():
+    """More (event, layer) segments than the index takes: refused after the seed fit has been captured on the
+    graph's branch, which the capture still has to join."""
+    import ctypes as C
+    b = _batch(64, n_events=3)
+    cfg = tkf.default_config(n_eta_bins=2, n_phi_bins=2, eta_bin_w=2.0)
+    ctx = tkf.Context(cfg)
+    L, n, many = cfg.n_layers, b.n_tracks, (1 << 22) // cfg.n_layers + 1
+    dh = device_hits(b)
+    sh = torch.as_tensor(np.ascontiguousarray(b.trk_hits[:, :3].T), dtype=torch.int32, device="cuda")
+    se = torch.as_tensor(b.trk_event, dtype=torch.int32, device="cuda")
+    pipe = tkf.DevicePipeline(ctx, b.n_hits, many, n, use_graph=True)
+    hs = dh.struct()
+    off = torch.cat([dh.event_off, dh.event_off[-1:].repeat(many - b.n_events)])
+    hs.event_off, hs.n_events = off.data_ptr(), many
+    for _ in range(2):
+        code = tkf.lib().tkf_pipeline_run(pipe.handle, C.byref(hs), C.c_void_p(sh.data_ptr()), C.c_void_p(se.data_ptr()), n, None)
+        assert code == tkf.ERR_INVALID
+        built, final = _direct(ctx, b, dh, sh, se)
+    pipe.run(dh, sh, se, n)
+    torch.cuda.synchronize()
+    bt, ft = _pipe_out(pipe, L, n)
+    assert torch.equal(bt["hit_idx"], built.hit_idx) and torch.equal(ft["par"], final.par) and torch.equal(ft["cov"], final.cov)
