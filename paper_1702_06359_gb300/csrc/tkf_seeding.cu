@@ -27,6 +27,7 @@
 
 #include "internal.h"
 #include "kf_math.cuh"
+#include "seed_window.cuh"
 
 using namespace tkf;
 
@@ -44,7 +45,7 @@ struct SeedGeom {
     float zv, d0, dz, w3, z3;
     float lim01, lim12, lim23;  // transverse chord limits 2 (R_{l+1} - R_l)
     float hit_dr;
-    float inv_lo[2];  // 1 / (R - hit_dr) of layers 2 and 3
+    SeedWindows win;
     float aspect[2];  // z extent of a layer-2 / layer-3 window over its phi extent
     int confirm;
 };
@@ -368,13 +369,6 @@ __device__ __forceinline__ RowPair row_pair(const int *__restrict__ tab, const S
     return w;
 }
 
-// asin(x) for a window's centre: the series to x^7 is within 4e-6 below 0.35
-__device__ __forceinline__ float asin_near(float x)
-{
-    const float q = x * x;
-    return fabsf(x) < 0.35f ? x * (1.f + q * (1.f / 6.f + q * (3.f / 40.f + q * (15.f / 336.f)))) : asinf(x);
-}
-
 // Ranges of layer-1 positions a lane has ahead of it, refilled kRanges at a time.
 constexpr int kRanges = 10;
 // Queues of one warp: layer-2 hits within a pair's chord and z cuts waiting for the circle through
@@ -477,9 +471,7 @@ k_seed_find(const SeedGeom g, const float4 *__restrict__ hxyzi, const int *__res
             const float zc_lo = fminf(az * rlo / ra - g.zv * (rlo / ra - 1.f), az * rhi / ra - g.zv * (rhi / ra - 1.f));
             const float zc_hi = fmaxf(az * rlo / ra + g.zv * (rlo / ra - 1.f), az * rhi / ra + g.zv * (rhi / ra - 1.f));
             eta_bins(g, R1, zc_lo - zpad, zc_hi + zpad, row, row_end);
-            const float s1 = g.kmax * rhi * 0.5f;
-            const float half = s1 >= 1.f ? 4.f : asinf(s1) - asinf(g.kmax * ra * 0.5f) + 2e-3f;
-            const PhiWin w1 = phi_window(g, pha, half);
+            const PhiWin w1 = phi_window(g, pha, half_layer1(g.win, rhi, ra));
             q.win[lane] = make_int4(w1.lo[0], w1.hi[0], w1.lo[1], w1.hi[1]);
             row += lane % G;
         }
@@ -512,56 +504,50 @@ k_seed_find(const SeedGeom g, const float4 *__restrict__ hxyzi, const int *__res
                     const float rb = sqrtf(dot2(B.y, B.y, B.x, B.x)), rc = Cc.w;
                     if (rc != rb) {
                         const float slope23 = (Cc.z - B.z) / (rc - rb);
-                        // where the circle crosses r = R3 nearest to c: its centre is U = a + rho n, and
-                        // the crossing lies along U at (R3^2 + 2 rho d0) / (2 |U|) (|U|^2 - rho^2 = 2 rho d0)
-                        const float rho = 1.f / kap;
-                        const float ux = A.x + rho * nx, uy = A.y + rho * ny;
-                        const float D = sqrtf(ux * ux + uy * uy);
-                        const float R3 = g.R[3];
-                        const float along = (R3 * R3 + 2.f * rho * d0) / (2.f * D);
-                        const float h2 = R3 * R3 - along * along;
-                        if (h2 >= 0.f) {
-                            const float h = sqrtf(h2), ex = ux / D, ey = uy / D;
+                        const float half = half_layer3(g.win, kap, d0), R3 = g.R[3];
+                        float ph3 = 0.f;
+                        if (half < kWholeRow) {
+                            // where the circle crosses r = R3 nearest to c: its centre is U = a + rho n, and
+                            // the crossing lies along U at (R3^2 + 2 rho d0) / (2 |U|) (|U|^2 - rho^2 = 2 rho d0)
+                            const float rho = 1.f / kap;
+                            const float ux = A.x + rho * nx, uy = A.y + rho * ny;
+                            const float D = sqrtf(ux * ux + uy * uy);
+                            const float along = (R3 * R3 + 2.f * rho * d0) / (2.f * D);
+                            const float h = sqrtf(fmaxf(R3 * R3 - along * along, 0.f)), ex = ux / D, ey = uy / D;
                             const float px1 = along * ex - h * ey, py1 = along * ey + h * ex;
                             const float px2 = along * ex + h * ey, py2 = along * ey - h * ex;
                             const bool near1 = (px1 - Cc.x) * (px1 - Cc.x) + (py1 - Cc.y) * (py1 - Cc.y) <=
                                                (px2 - Cc.x) * (px2 - Cc.x) + (py2 - Cc.y) * (py2 - Cc.y);
-                            const float ph3 = atan2f(near1 ? py1 : py2, near1 ? px1 : px2);
-                            const float zc3 = B.z + slope23 * (R3 - rb);
-                            const float wz = g.z3 + 1e-3f + 1e-5f * fabsf(zc3) + g.hit_dr * fabsf(slope23);
-                            const SeedCells c3 = load_cells(&cells[q.grid[ts] + 1]);
-                            // a hit within w3 of the circle lies within about w3 / sqrt(1 - x^2) of the
-                            // crossing, as above (random circles reach 0.77 of it)
-                            const float x = kap * (R3 + g.hit_dr) * 0.5f, wk = 1.f / (1.f - x * x);
-                            const float half = x < 0.9f ? (1.25f * g.w3 * wk + 0.005f) * g.inv_lo[1] +
-                                                              g.hit_dr * (0.75f * kap * wk + 1.25f * g.d0 / (R3 * R3)) + 3e-4f
-                                                        : 4.f;
-                            const GridWin w3 = grid_window(c3, zc3, wz, ph3, half);
-                            float c3s = kInf;
-                            for (int r = w3.r0; r <= w3.r1; r += 2) {
-                                RowPair rp = row_pair(tab, c3, r, w3.r1, w3.lo0, w3.hi0);
-                                for (int i = 0;; ++i) {
-                                    if (i >= rp.n) {  // the window's second run, if it has one
-                                        if (w3.hi1 < 0 || rp.second) break;
-                                        rp = row_pair(tab, c3, r, w3.r1, 0, w3.hi1);
-                                        rp.second = true;
-                                        i = -1;
-                                        continue;
-                                    }
-                                    const float4 E = gxyzr[rp.at(i)];
-                                    const float d23x = E.x - Cc.x, d23y = E.y - Cc.y;
-                                    if (!(sqrtf(d23x * d23x + d23y * d23y) <= g.lim23)) continue;
-                                    const float qx = E.x - A.x, qy = E.y - A.y;
-                                    const float f3 = kap * dot2(qx, qx, qy, qy) * 0.5f - dot2(qx, nx, qy, ny);
-                                    const float re = E.w;
-                                    const float dz3 = E.z - (B.z + slope23 * (re - rb));
-                                    if (!(fabsf(f3) <= g.w3) || !(fabsf(dz3) <= g.z3)) continue;
-                                    const float pu = f3 / g.w3, pv = dz3 / g.z3;
-                                    c3s = fminf(c3s, dot2(pu, pu, pv, pv));
-                                }
-                            }
-                            if (c3s < kInf) s = s2 + c3s;
+                            ph3 = atan2f(near1 ? py1 : py2, near1 ? px1 : px2);
                         }
+                        const float zc3 = B.z + slope23 * (R3 - rb);
+                        const float wz = g.z3 + 1e-3f + 1e-5f * fabsf(zc3) + g.hit_dr * fabsf(slope23);
+                        const SeedCells c3 = load_cells(&cells[q.grid[ts] + 1]);
+                        const GridWin w3 = grid_window(c3, zc3, wz, ph3, half);
+                        float c3s = kInf;
+                        for (int r = w3.r0; r <= w3.r1; r += 2) {
+                            RowPair rp = row_pair(tab, c3, r, w3.r1, w3.lo0, w3.hi0);
+                            for (int i = 0;; ++i) {
+                                if (i >= rp.n) {  // the window's second run, if it has one
+                                    if (w3.hi1 < 0 || rp.second) break;
+                                    rp = row_pair(tab, c3, r, w3.r1, 0, w3.hi1);
+                                    rp.second = true;
+                                    i = -1;
+                                    continue;
+                                }
+                                const float4 E = gxyzr[rp.at(i)];
+                                const float d23x = E.x - Cc.x, d23y = E.y - Cc.y;
+                                if (!(sqrtf(d23x * d23x + d23y * d23y) <= g.lim23)) continue;
+                                const float qx = E.x - A.x, qy = E.y - A.y;
+                                const float f3 = kap * dot2(qx, qx, qy, qy) * 0.5f - dot2(qx, nx, qy, ny);
+                                const float re = E.w;
+                                const float dz3 = E.z - (B.z + slope23 * (re - rb));
+                                if (!(fabsf(f3) <= g.w3) || !(fabsf(dz3) <= g.z3)) continue;
+                                const float pu = f3 / g.w3, pv = dz3 / g.z3;
+                                c3s = fminf(c3s, dot2(pu, pu, pv, pv));
+                            }
+                        }
+                        if (c3s < kInf) s = s2 + c3s;
                     }
                 }
             }
@@ -676,25 +662,16 @@ k_seed_find(const SeedGeom g, const float4 *__restrict__ hxyzi, const int *__res
                 }
             }
             // its layer-2 window: z along the r-z line of a and b, phi around the crossing of the circle
-            // through the beam line, a and b, widened by the d0 cut's lever arm
+            // through the beam line, a and b
             GridWin w2;
             w2.r0 = 0; w2.r1 = -1; w2.lo0 = 0; w2.hi0 = 0; w2.hi1 = -1; w2.back = 0;
             if (pass) {
                 const float R2 = g.R[2];
                 const float zc = az + slope * (R2 - ra);
                 const float wz = g.dz + 1e-3f + 1e-5f * fabsf(zc) + g.hit_dr * fabsf(slope);
-                // The circles through a and b that pass within d0 of the beam line differ from the one
-                // through it by d0 (R2 - ra) (R2 - rb) / (ra rb) at R2, to first order in d0 and in
-                // x^2 = (k01 R2 / 2)^2, and turn by k01 / (2 sqrt(1 - x^2)) per cm of hit_dr.  Random
-                // circles (curvatures up to x = 0.9, d0 up to 1.5 cm) reach 0.86 of this half width.
-                float half = 4.f, mid = pha;
-                const float x = fabsf(k01) * (R2 + g.hit_dr) * 0.5f;
-                if (x < 0.9f) {
-                    const float lever = (R2 + g.hit_dr - ra) * (R2 + g.hit_dr - rb) / (ra * rb), w = 1.f / (1.f - x * x);
-                    half = (1.25f * g.d0 * lever * w + 0.005f) * g.inv_lo[0] + 0.75f * g.hit_dr * fabsf(k01) * w + 3e-4f;
-                    mid = pha + asin_near(k01 * R2 * 0.5f) - asin_near(k01 * ra * 0.5f);
-                }
-                w2 = grid_window(c2, zc, wz, mid, half);
+                float mid;
+                const float half = half_layer2(g.win, ra, rb, k01, mid);
+                w2 = grid_window(c2, zc, wz, pha + mid, half);
             }
             // two rows at a time, the few hits of both in one sequence
             while (__any_sync(full, w2.r0 <= w2.r1)) {
@@ -960,7 +937,7 @@ extern "C" int tkf_find_seeds(tkf_ctx *ctx, const tkf_hit_index *idx, const tkf_
     g.confirm = cuts->confirm != 0;
     // z extent over phi extent of the nominal windows (the grids' cells are shaped like them)
     const double lever = (c.radius[2] - c.radius[0]) * (c.radius[2] - c.radius[1]) / (c.radius[0] * c.radius[1]);
-    for (int k = 0; k < 2; ++k) g.inv_lo[k] = (float)(1.0 / (c.radius[2 + k] - c.hit_dr));
+    g.win = seed_windows(c.radius, c.hit_dr, g.kmax, cuts->d0_max, cuts->conf_rphi);
     g.aspect[0] = (float)((cuts->dz_max + 1e-3) / ((1.25 * cuts->d0_max * lever + 0.005) / c.radius[2] + 3e-4));
     g.aspect[1] = (float)((cuts->conf_z + 1e-3) / ((1.25 * cuts->conf_rphi + 0.005) / c.radius[3] + 3e-4));
     SeedCells *cells = (SeedCells *)ctx->seed_cells;

@@ -74,3 +74,43 @@ def test_windows_lose_no_seed_of_the_brute_force_search(pt_min, d0, hit_dr):
                 assert mine is not None and mine[:2] == (o + p["h1"], o + p["h2"]) and abs(mine[2] - p["score"]) <= 2e-4
                 found += 1
     assert found >= 100
+
+
+# cuts so wide that circles far from the one through the beam line pass, on layers of unequal steps (16 - 6 > 6,
+# where the chord cut leaves a circle's far branch), with and without the confirmation
+@pytest.mark.parametrize("confirm", [0, 1])
+@pytest.mark.parametrize("radii,pt_min,d0", [((3, 6, 16, 25), 0.06, 1.5), ((4, 8, 12, 16), 0.06, 1.0), ((4, 8, 20, 24), 0.1, 1.0),
+                                             ((3, 10, 13, 17), 0.2, 0.5)])
+def test_wide_cuts_on_random_hits_lose_no_seed(radii, pt_min, d0, confirm):
+    rng = np.random.default_rng(int(100 * d0) + confirm)
+    n_ev, per = 40, 24
+    layer = np.tile(np.repeat(np.arange(4), per), n_ev)
+    r, phi = np.array(radii, float)[layer], rng.uniform(-np.pi, np.pi, len(layer))
+    x, y, z = (a.astype(np.float32) for a in (r * np.cos(phi), r * np.sin(phi), rng.uniform(-1, 1, len(layer))))
+    t = lambda a: torch.as_tensor(a, device="cuda")  # noqa: E731
+    v = torch.full((len(layer),), 1e-4, device="cuda")
+    off = np.arange(n_ev + 1, dtype=np.int32) * 4 * per
+    cuts = tkf.default_seed_cuts(pt_min=pt_min, d0_max=d0, z_vertex=100.0, dz_max=50.0, conf_rphi=1.0, conf_z=50.0, confirm=confirm)
+    h, _, s = (a.cpu().numpy() for a in _seeds(tkf.DeviceHits(t(x), t(y), t(z), v, v, t(layer.astype(np.int32)), t(off)), cuts,
+                                               len(layer), n_layers=4, radius=radii))
+    got = {int(a): (int(p), int(q), float(w)) for a, p, q, w in zip(h[0], h[1], h[2], s)}
+    det = Detector(radii=tuple(float(r) for r in radii), x_over_x0=(0.03,) * 4)
+    g = O.make_geom(det)
+    co = O.SeedCuts(*(getattr(cuts, k) for k in ("pt_min", "kappa_slack", "z_vertex", "d0_max", "dz_max", "conf_rphi", "conf_z")), confirm)
+    found = 0
+    for ev in range(n_ev):
+        sl = slice(off[ev], off[ev + 1])
+        hits = np.zeros(4 * per, O.HIT_DTYPE)
+        for k, a in (("x", x), ("y", y), ("z", z), ("layer", layer)):
+            hits[k] = a[sl]
+        picks = O.find_seeds(g, co, hits)
+        for a in range(per):
+            p, mine = picks[a], got.get(int(off[ev]) + a)
+            if p["margin"] < 1e-4 or p["gap"] < 1e-4:
+                continue
+            if p["h1"] < 0:
+                assert mine is None
+            else:
+                assert mine is not None and mine[:2] == (off[ev] + p["h1"], off[ev] + p["h2"]) and abs(mine[2] - p["score"]) <= 2e-4
+                found += 1
+    assert found >= 100
