@@ -50,10 +50,11 @@ enum tkf_status_code {
 };
 
 /* Arithmetic of the KF steps (Sec. 3.2: the update's numerical stability).  FP32: everything
- * in float.  MIXED: float, except the innovation covariance, its inverse, the gain and the
- * covariance update, done on pairs of floats (about 46 bits; in double, in the Joseph form, where
- * a variance shrinks by more than 2^16 or a value leaves the pairs' range) and rounded back to
- * what double gives (the state update applies the rounded gain in float).  FP64: everything in double (track arrays hold double). */
+ * in float.  MIXED: float, except the innovation covariance, its inverse, the gain K and the
+ * covariance update, done on pairs of floats (about 46 bits) as P - K B, each element rounded to float
+ * once; the pairs' own errors add at most a quarter of that rounding to a variance.  Where a variance
+ * shrinks by more than 2^16 or a value leaves the pairs' range: in double, in the Joseph form.  The
+ * state update applies the rounded gain in float.  FP64: everything in double (track arrays hold double). */
 enum tkf_precision { TKF_FP32 = 0, TKF_MIXED = 1, TKF_FP64 = 2 };
 
 /* Per-track status written to tkf_tracks.nhits when a track fails (nhits < 0). */
