@@ -53,7 +53,6 @@ TKF_PAIR pair32 two_prod(float a, float b)
     const float p = mul_rn(a, b);
     return {p, fma_rn(a, b, -p)};
 }
-TKF_PAIR pair32 neg(pair32 a) { return {-a.h, -a.l}; }
 TKF_PAIR pair32 add(pair32 a, pair32 b)
 {
     const pair32 s = two_sum(a.h, b.h);
