@@ -151,7 +151,7 @@ template <> struct Lim<float> {
     static constexpr float converged = 1e-6f;
 };
 template <> struct Lim<double> {
-    // with two terms more than float's series below: within 2^-53 up to here, so that a warp's tracks
+    // with one term more than float's series below: within 2^-53 up to here, so that a warp's tracks
     // above 0.2 GeV between layers 4 cm apart all take the series (sincos of some lanes and the series
     // of the others both ran before)
     static constexpr double series = 0.25;

@@ -63,7 +63,7 @@ TKF_WIN float win_rsqrt(float x)
 #endif
 }
 
-// Half width of the layer-1 window around the azimuth of a first hit at radius ra; R1: its outer radius.
+// Half width of the layer-1 window around the azimuth of a first hit at radius ra; rhi: the layer's outer radius.
 TKF_WIN float half_layer1(const SeedWindows &g, float rhi, float ra)
 {
     const float s = g.kmax * rhi * 0.5f;
