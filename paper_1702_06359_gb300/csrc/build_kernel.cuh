@@ -38,8 +38,6 @@ namespace tkf {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr unsigned kEmpty32 = 0xFFFFFFFFu;
-constexpr int kFirstThreads = 128;                 // of k_first_scan's blocks
-constexpr int kFirstWide = kFirstThreads * 152;  // seeds from which such blocks reach every SM
 
 template <class R> __device__ __forceinline__ R pick(float f, double d);
 template <> __device__ __forceinline__ float pick<float>(float f, double) { return f; }
@@ -864,10 +862,7 @@ cudaError_t launch_build_t(const BuildArgs &a, int nmax, int grid, cudaStream_t 
         default: ff = TKF_F(16); break;
         }
 #undef TKF_F
-        // blocks of one warp where blocks of four would leave SMs without one: an event of 1000 tracks 82.9 ->
-        // 78.4 us for its step, of 3000 and 5000 the same; 2.6 M seeds 8.371 ms with 128 threads, 8.383 with 32
-        const int fth = a.n_seeds < kFirstWide ? 32 : kFirstThreads;
-        const cudaError_t e = go(ff, (a.n_seeds + fth - 1) / fth, fth);
+        const cudaError_t e = go(ff, (a.n_seeds + a.first_threads - 1) / a.first_threads, a.first_threads);
         if (e != cudaSuccess) return e;
     }
     return go(fn, grid, threads);

@@ -55,7 +55,9 @@ struct BuildArgs {
     int *f_hit;
     int *tile_counter;
     int *err;
+    int first_threads;  // of k_first_scan's blocks
 };
+constexpr int kFirstThreads = 128;  // at most
 
 // Launchers of the build kernel, one translation unit per precision.  `nmax` is the
 // compile-time candidate capacity (1, 4, 6, 10 or 16) >= a.ncand.  `occupancy` (if not
