@@ -1106,9 +1106,10 @@ cudaError_t launch_segment_index(const IndexGeom &g, const tkf_hits &h, int sm_c
     auto take = [&](auto kern, int threads, size_t smem) {
         const int hi = segment_cap(g.n_bins, smem);
         if (e == cudaSuccess) e = launch_next(kern, n_segs, threads, smem, s, g, h, x, lo, hi);
-        lo = std::max(hi, -1);
+        lo = hi;
     };
-    if ((int)n_segs > sm_count) take(k_index_segment<kSegThreads, 2, false>, kSegThreads, kSegSmem);
+    // (from some 3600 bins on the counters alone fill the smaller class's share)
+    if ((int)n_segs > sm_count && segment_cap(g.n_bins, kSegSmem) > 0) take(k_index_segment<kSegThreads, 2, false>, kSegThreads, kSegSmem);
     take(k_index_segment<kSegThreadsBig, 1, true>, kSegThreadsBig, kSegSmemBig);
     return e;
 }

@@ -158,3 +158,29 @@ def test_dense_bins_and_large_segments_have_the_index_of_their_cells(n_eta, n_ph
     vmax = np.zeros((E * L, 2), np.float32)
     np.maximum.at(vmax, ev * L + layer, np.stack(f[3:], 1))
     assert np.array_equal(got["vmax"].view(np.float32), vmax)
+
+
+# 40 events run in two size classes, ten in one; with 60 x 63 bins the smaller class has no room for hits
+@pytest.mark.parametrize("n_eta,n_phi", [(40, 63), (57, 62), (60, 63), (64, 64)])
+def test_size_classes_give_the_same_index(n_eta, n_phi):
+    per = [[int(900 * (1 + (3 * e + l) % 11)) if l < 4 else 10 * l for l in range(L)] for e in range(40)]
+    f, layer, off = _hits(per, "grouped", False)
+    nb = n_eta * n_phi
+    ctx = tkf.Context(_config(n_eta, n_phi, False))
+
+    def index(e0, e1):
+        a, b = off[e0], off[e1]
+        idx = ctx.build_hit_index(_device([x[a:b] for x in f], layer[a:b], off[e0:e1 + 1] - a))
+        ctx.sync_status()
+        got = _planes(idx.view(), int(b - a), (e1 - e0) * L, nb, e1 - e0)
+        idx.free()
+        return got
+    whole = index(0, 40)
+    for e0 in range(0, 40, 10):
+        part, a, b, s = index(e0, e0 + 10), int(off[e0]), int(off[e0 + 10]), slice(e0 * L, (e0 + 10) * L)
+        for k in ("xyzi", "var"):
+            assert torch.equal(whole[k][a:b], part[k])
+        assert torch.equal(whole["pos"][a:b], part["pos"] + a)
+        assert torch.equal(whole["off"][e0 * L * nb:(e0 + 10) * L * nb + 1], part["off"] + a)
+        assert torch.equal(whole["sub"][e0 * L * nb:(e0 + 10) * L * nb], part["sub"]) and torch.equal(whole["vmax"][s], part["vmax"])
+    ctx.close()
