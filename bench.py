@@ -1099,7 +1099,7 @@ def main():
                    "batches"
                    % (b.n_events, a.e2e_slots, a.e2e_batch)}
 
-    # ---------------- the same batched step in MIXED precision (FP64 inverse + Joseph update)
+    # ---------------- the same batched step in MIXED precision (inverse, gain and covariance on pairs of floats)
     mixed = None
     if a.mixed:
         mctx = tkf.Context(tkf.default_config(seed_order=a.seed_order, precision=tkf.MIXED,
@@ -1129,8 +1129,8 @@ def main():
                               "note": "the FP32 form's operations, with the updates' double arithmetic on pairs of "
                                       "floats (one operation per instruction); each block's updates run packed into "
                                       "full warps"},
-                 "precision": "mixed: FP32 propagation, window and chi2; innovation inverse and Joseph update on pairs "
-                              "of floats (48 bits)",
+                 "precision": "mixed: FP32 propagation, window and chi2; innovation inverse, gain and covariance update "
+                              "P - K B on pairs of floats (about 46 bits)",
                  "seeds_per_warp_tile": best_tile}
         mpipe.close()
         mctx.close()

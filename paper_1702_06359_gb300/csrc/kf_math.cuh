@@ -770,8 +770,9 @@ template <bool kDisk> __device__ __noinline__ MixedUpdate mixed_update_double(Mi
 
 // The mixed-precision update: kalman_update<double, float> with its double arithmetic done on
 // pairs of floats (pair_f32.cuh), because the double units bound every mixed kernel: a fit of
-// 163 k tracks spent 0.515 ms on ten layers at the full double rate, and takes 0.068 ms on pairs.  With the gain good to 2^-45 the Joseph form's second product,
-// (B^T - K S) K^T, is below that too, and P' = P - K B is formed with one rounding per element.
+// 163 k tracks spent 0.515 ms on ten layers at the full double rate, and takes 0.068 ms on pairs.
+// With the gain good to 2^-45 the Joseph form's second product, (B^T - K S) K^T, is below that too,
+// and P' = P - K B is formed with one rounding per element.
 //
 // What the roundings leave in P' is about 2^-45 of P, so the update may shrink a variance by
 // kPairShrink = 2^16 at most (S / V, times 1 / (1 - rho^2) of the correlation in S) for them to

@@ -413,8 +413,8 @@ __device__ __forceinline__ SeedCells load_cells(const SeedCells *p)
 // What bounds it: instruction issue and the latency of gathered 16-byte reads together (55 % issue
 // active, half of the L1 sectors hit).  On the 160-event batch (880 k first hits, 48 M passing
 // pairs) it takes 2.3 M steps of about 480 instructions; reading the layer-2 windows from the hit
-// index took 2.9 G instructions, this 1.1 G: 4.13 -> 1.85 ms, 640 events 16.0 -> 7.0 ms, one
-// event of 3000 tracks 169 -> 57 us.  5 blocks of 128 threads per SM (94 registers): 4 blocks 2.13
+// index took 2.9 G instructions, this 1.1 G: 4.13 -> 1.83 ms, 640 events 16.0 -> 7.0 ms, one
+// event of 3000 tracks 169 -> 57 us.  5 blocks of 128 threads per SM (88 registers): 4 blocks 2.13
 // ms, 6 1.95 ms (the L1 that is left to the hits shrinks with the queues' shared memory); a pair's
 // hit loaded one step ahead 1.91 ms.
 constexpr int kFindBlocksPerSM = 5;
