@@ -475,11 +475,11 @@ __host__ __device__ __forceinline__ int whole_cap(int n_bins)
     return n < 65535 ? n : 65535;
 }
 // A segment of more hits is taken in parts, each some of its bins: a counter for each bin of the segment,
-// the part's sixteenths, 8 bytes for each of the part's hits.
+// and, of the part, the sixteenths and 4 bytes for each hit.
 __host__ __device__ __forceinline__ int part_bin_words(int n_bins) { return (n_bins + 4) / 4; }
-__host__ __device__ __forceinline__ int part_cap(int n_bins)
+__device__ __forceinline__ bool part_fits(int n_bins, int bins, int hits)
 {
-    return ((int)kSegSmemBig - 16 * (part_bin_words(n_bins) + seg_words(n_bins))) / 8;
+    return hits < 65536 && 16 * (part_bin_words(n_bins) + seg_words(bins)) + 4 * hits <= (int)kSegSmemBig;
 }
 
 // The layers of hits i .. i + 3 (-1 outside h0 .. h1 - 1), as one word where the array is aligned to it.
@@ -770,14 +770,14 @@ template <int T> __device__ __forceinline__ void fill_free(const SegIndex &x, in
 
 // A segment too large for the keys of its hits in shared memory, by one block: they wait in pos_of_hit.
 // Up to 65535 hits it is ordered at once, as a smaller one.  Of a larger one the hits per bin are counted
-// first; then its bins are taken in parts, whose hits are collected and ordered.  A bin that is too large by
-// itself is ordered by words in global memory.  What bounds it: one block's scattered accesses, 32
-// bytes for 4.  A layer of 40 k / 110 k hits beside nine of 4 k: 126 / 689 us, ten layers of 67 k / 270 k 0.39 /
-// 3.6 ms; by the multi-launch kernels 166 / 574 us and 0.34 / 75.6 ms, with all hits ordered by words 1183 /
+// first; then its bins are taken in parts, each ordered like that.  A bin that is too large by itself is
+// ordered by words in global memory.  What bounds it: one block's scattered accesses, 32
+// bytes for 4.  A layer of 40 k / 110 k hits beside nine of 4 k: 126 / 597 us, ten layers of 67 k / 270 k 0.34 /
+// 3.0 ms; by the multi-launch kernels 166 / 574 us and 0.34 / 75.6 ms, with all hits ordered by words 1183 /
 // 9193 us and 3.5 / 57 ms.  Measured and not taken: parts for other blocks, each binning the whole segment (109 /
 // 227 us, 0.20 / 1.6 ms), because the blocks that look for parts made every batch slower (20 events
 // 44.2 -> 46.8 us, 512 events 720 -> 728); hits placed into their bins and ordered there in place 0.82 ms for
-// the layer of 110 k.
+// the layer of 110 k, parts whose hits are listed and fetched by their numbers 0.69 ms.
 template <int T>
 __device__ __noinline__ void segment_large(const IndexGeom &g, const tkf_hits &h, const SegIndex &x, int seg, int cnt,
                                            int base, uint4 *s_words, int *s_part, int *s_mu, int *s_mv)
@@ -791,12 +791,9 @@ __device__ __noinline__ void segment_large(const IndexGeom &g, const tkf_hits &h
     const float rl = g.radius[l];
     const bool disk = (g.disk_mask >> l) & 1u;
     const size_t b0 = (size_t)seg * nb;
-    const int cap = part_cap(nb);
     int *s_bin = (int *)s_words;  // [nb + 1]
     uint4 *s_cells = s_words + part_bin_words(nb);
     unsigned *s_cell = (unsigned *)s_cells;
-    int *s_id = (int *)(s_cells + seg_words(nb));
-    unsigned short *s_key = (unsigned short *)(s_id + cap), *s_ord = s_key + cap;
     float mu = 0.f, mv = 0.f;
     auto done = [&]() {
         const int2 most = block_max(mu, mv, s_mu, s_mv);
@@ -878,80 +875,80 @@ __device__ __noinline__ void segment_large(const IndexGeom &g, const tkf_hits &h
         // the part: bins first .. end - 1, and their hits, own of them from position a of the segment on
         const int a = s_bin[first];
         end = first + 1;
-        for (int hi = nb; end < hi;) {  // the most bins whose hits fit, or one
+        for (int hi = nb; end < hi;) {  // the most bins that fit, or one
             const int mid = (end + hi + 1) >> 1;
-            if (s_bin[mid] - a <= cap) end = mid; else hi = mid - 1;
+            if (part_fits(nb, mid - first, s_bin[mid] - a)) end = mid; else hi = mid - 1;
         }
-        const int own = s_bin[end] - a;
-        // f(hit's place in the segment, hit, key, its number) for the part's hits, numbered from s_n on
-        auto each_own = [&](auto f) {
-            constexpr int U = 4;
-            for (int q0 = 0; q0 < cnt; q0 += U * T) {  // every thread takes every turn
-                int i[U], key[U], total = 0;
-                unsigned in[U];
+        const int own = s_bin[end] - a, nw = seg_words(end - first);
+        // whether a hit with key `key` in pos_of_hit is the part's (placed ones have none); its sixteenth k
+        auto is_own = [&](int key, unsigned &k) {
+            k = (unsigned)(key & ~kWaiting) - first * kSubBins;  // (wraps below the part)
+            return key < 0 && k < (unsigned)(end - first) * kSubBins;
+        };
+        auto each_own = [&](auto f) {  // f(hit's place in the segment, hit, its sixteenth in the part)
+            constexpr int U = 8;
+            for (int j0 = tid; j0 < cnt; j0 += U * T) {
+                int i[U], key[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    i[u] = at(min(q0 + u * T + tid, cnt - 1));
+                    i[u] = at(min(j0 + u * T, cnt - 1));
                     key[u] = x.pos_of_hit[i[u]];
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const unsigned k = (unsigned)(key[u] & ~kWaiting);
-                    in[u] = __ballot_sync(full, q0 + u * T + tid < cnt && key[u] < 0 && k >= (unsigned)first * kSubBins &&
-                                                    k < (unsigned)end * kSubBins);
-                    total += __popc(in[u]);
-                }
-                int m = 0;  // (one number a hit taken from s_n: 17 k of them in turn)
-                if (lane == 0 && total > 0) m = atomicAdd(&s_n, total);
-                m = __shfl_sync(full, m, 0);
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if (in[u] >> lane & 1u)
-                        f(q0 + u * T + tid, i[u], (unsigned)(key[u] & ~kWaiting), m + __popc(in[u] & ((1u << lane) - 1u)));
-                    m += __popc(in[u]);
+                    unsigned k;
+                    if (j0 + u * T < cnt && is_own(key[u], k)) f(j0 + u * T, i[u], k);
                 }
             }
         };
-        if (tid == 0) s_n = 0;
-        if (own <= cap) {
-            const int nw = seg_words(end - first);
+        if (part_fits(nb, end - first, own)) {
+            int *s_place = (int *)(s_cells + nw);
             for (int k = tid; k < nw; k += T) s_cells[k] = make_uint4(0u, 0u, 0u, 0u);
             __syncthreads();
-            // (2) the part's hits, in no order: place in the segment and sixteenth
-            each_own([&](int j, int, unsigned key, int m) {
-                key -= first * kSubBins;
-                s_id[m] = j;
-                s_key[m] = (unsigned short)key;
-                atomicAdd(&s_cell[key >> 1], key & 1 ? 0x10000u : 1u);
-            });
+            // (2) as for a smaller segment, each pass over all of its hits in the order of the input: taking the
+            // part's own by a list would fetch 32 bytes for 4
+            each_own([&](int, int, unsigned k) { atomicAdd(&s_cell[k >> 1], k & 1 ? 0x10000u : 1u); });
             __syncthreads();
             cell_ends<T>(s_cells, nw, s_part);
-            for (int m = tid; m < own; m += T) {
-                const unsigned key = s_key[m], sh = 16 * (key & 1);
-                const unsigned old = atomicSub(&s_cell[key >> 1], 1u << sh);
-                s_ord[((old >> sh) & 0xFFFFu) - 1] = (unsigned short)m;
-            }
+            each_own([&](int j, int, unsigned k) {
+                const unsigned sh = 16 * (k & 1), old = atomicSub(&s_cell[k >> 1], 1u << sh);
+                s_place[((old >> sh) & 0xFFFFu) - 1] = j;
+            });
             __syncthreads();
             for (int b = first + tid; b < end; b += T) {
                 unsigned rel;
                 x.bin_sub[b0 + b] = bin_table(s_cells, b - first, rel);
                 x.bin_off[b0 + b] = base + a + (int)rel;
             }
-            // (3) to their places: a sixteenth's hits in the order of their ids
-            for_hits<T>(h, [&](int m) { return at(s_id[m]); }, own, [&](int m, float hx, float hy, float hz) {
-                const unsigned key = s_key[m];
-                const int a0 = (int)half16(s_cell, key), a1 = (int)half16(s_cell, key + 1), j = s_id[m];
-                int pos = base + a + a0;
-                if (a1 - a0 > 1)
-                    for (int t = a0; t < a1; ++t) pos += s_id[s_ord[t]] < j;
-                const int i = at(j);
-                const float vu = h.var_u[i], vv = h.var_v[i];
-                x.hxyzi[pos] = make_float4(hx, hy, hz, __int_as_float(i - h0));
-                x.hvar[pos] = make_float2(vu, vv);
-                x.pos_of_hit[i] = pos;
-                mu = fmaxf(mu, vu);
-                mv = fmaxf(mv, vv);
-            });
+            constexpr int U = 4;
+            for (int j0 = tid; j0 < cnt; j0 += U * T) {
+                int i[U], key[U];
+                float hx[U], hy[U], hz[U], vu[U], vv[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    i[u] = at(min(j0 + u * T, cnt - 1));
+                    key[u] = x.pos_of_hit[i[u]];
+                    hx[u] = h.x[i[u]];
+                    hy[u] = h.y[i[u]];
+                    hz[u] = h.z[i[u]];
+                    vu[u] = h.var_u[i[u]];
+                    vv[u] = h.var_v[i[u]];
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    unsigned k;
+                    if (j0 + u * T >= cnt || !is_own(key[u], k)) continue;
+                    const int a0 = (int)half16(s_cell, k), a1 = (int)half16(s_cell, k + 1);
+                    int pos = base + a + a0;
+                    if (a1 - a0 > 1)
+                        for (int t = a0; t < a1; ++t) pos += s_place[t] < j0 + u * T;
+                    x.hxyzi[pos] = make_float4(hx[u], hy[u], hz[u], __int_as_float(i[u] - h0));
+                    x.hvar[pos] = make_float2(vu[u], vv[u]);
+                    x.pos_of_hit[i[u]] = pos;
+                    mu = fmaxf(mu, vu[u]);
+                    mv = fmaxf(mv, vv[u]);
+                }
+            }
         } else {  // one bin: words of sixteenth and id in its part of hvar
             // (the id whole: an event over the hit limit, which is reported, has ids beyond 23 bits, and two
             // words that compared equal would leave a position of the index unwritten)
@@ -959,15 +956,16 @@ __device__ __noinline__ void segment_large(const IndexGeom &g, const tkf_hits &h
             auto order_word = [&](unsigned key, int i) {
                 return ((unsigned long long)(key & (kSubBins - 1)) << 32) | (unsigned)(i - h0);
             };
+            if (tid == 0) s_n = 0;
             __syncthreads();
-            each_own([&](int, int i, unsigned key, int m) { g_ord[m] = order_word(key, i); });
+            each_own([&](int, int i, unsigned k) { g_ord[atomicAdd(&s_n, 1)] = order_word(k, i); });
             __syncthreads();
             if (tid == 0) {
                 x.bin_off[b0 + first] = base + a;
                 x.bin_sub[b0 + first] = make_uint4(~0u, ~0u, ~0u, ~0u);  // more than 255 hits
             }
-            each_own([&](int, int i, unsigned key, int) {
-                const unsigned long long word = order_word(key, i);
+            each_own([&](int, int i, unsigned k) {
+                const unsigned long long word = order_word(k, i);
                 int pos = base + a;
                 for (int t = 0; t < own; ++t) pos += g_ord[t] < word;
                 x.pos_of_hit[i] = pos;

@@ -61,7 +61,7 @@ def _config(n_eta, n_phi, disks):
 
 
 # hits of each layer: around the most that a block holds with its keys (37 697 with 2520 bins) and without
-# (65 535; 50 168 with 4096 bins), more (parts of 17 584 and 10 492), small and empty segments
+# (65 535; 50 168 with 4096 bins), more (in parts), small and empty segments
 MIXED = [65535, 65536, 25, 70001, 0, 50168, 50169, 37698, 1, 37697]
 EVEN = [17000] * L
 
